@@ -55,20 +55,20 @@ k_step(const Params<typename Store<PREC>::C> p, const typename Store<PREC>::T *_
             const bool ox = p.abb_x && (xs < 0 || xs >= p.nx);
             const bool oy = p.abb_y && (ys < 0 || ys >= p.ny);
             if (ox || oy) {
-                const C wx = xs < 0 ? p.phi_wall[0] : p.phi_wall[1];
-                const C wy = ys < 0 ? p.phi_wall[2] : p.phi_wall[3];
-                const C phiw = (ox && oy) ? C(0.5) * (wx + wy) : (ox ? wx : wy);
-                f[k] = wall_term<C, CONV, DIFF>(p, k, phiw) - S::ld(src + opp(k) * P, own, src_phi, wgt<C>(opp(k)));
+                f[k] = wall_value<PREC, C, CONV, DIFF>(p, k, ox, oy) - S::ld(src + opp(k) * P, own, src_phi, wgt<C>(opp(k)));
             }
         }
     }
 
     C phi;
+    // (FP32 with a per-node tensor keeps collide(): these are the forward states of the
+    // adjoint, whose gradient in u is a sum of cancelling terms that magnifies a change
+    // of the last bit)
     if (p.Afield)
-        collide<C, CONV, DIFF, true>(p, f, __ldg(p.Afield + own), __ldg(p.Afield + P + own), __ldg(p.Afield + 2 * P + own),
-                                     phi);
+        collide_stored<PREC == LBM_F32 ? LBM_BF16S : PREC, C, CONV, DIFF, true>(
+            p, f, __ldg(p.Afield + own), __ldg(p.Afield + P + own), __ldg(p.Afield + 2 * P + own), phi);
     else
-        collide<C, CONV, DIFF, false>(p, f, p.A3, p.A35, p.A5, phi);
+        collide_stored<PREC, C, CONV, DIFF, false>(p, f, p.A3, p.A35, p.A5, phi);
     S::store_cell(dst, dst_phi, P, own, f, phi);
 }
 

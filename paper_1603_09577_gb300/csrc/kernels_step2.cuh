@@ -72,10 +72,7 @@ __device__ __forceinline__ void pull_global(const Params<float> &p, const typena
                 const bool ox = p.abb_x && (xs < 0 || xs >= p.nx);
                 const bool oy = p.abb_y && (ys < 0 || ys >= p.ny);
                 if (ox || oy) {
-                    const float wx = xs < 0 ? p.phi_wall[0] : p.phi_wall[1];
-                    const float wy = ys < 0 ? p.phi_wall[2] : p.phi_wall[3];
-                    const float phiw = (ox && oy) ? 0.5f * (wx + wy) : (ox ? wx : wy);
-                    f[k] = wall_term<float, CONV, DIFF>(p, k, phiw) - S::ld(src + opp(k) * P, own, src_h, wgt<float>(opp(k)));
+                    f[k] = wall_value<PREC, float, CONV, DIFF>(p, k, ox, oy) - S::ld(src + opp(k) * P, own, src_h, wgt<float>(opp(k)));
                 }
             }
         }
@@ -98,12 +95,13 @@ __device__ __forceinline__ Params<F2> widen(const Params<float> &p)
     w.r0 = p.r0; w.r1 = p.r1; w.half_r0 = p.half_r0; w.inv_den = p.inv_den; w.inv_post = p.inv_post;
     w.has_src = p.has_src;
     w.Afield = nullptr;
+    w.k = coll_cast<F2>(p.k);
     return w;
 }
 
 // collide two nodes with one packed instruction stream; NODE_K: A3, A35, A5
 // are the nodes' blocks (per-node tensor field), else the constant block of pw
-template <int CONV, int DIFF, bool NODE_K>
+template <int PREC, int CONV, int DIFF, bool NODE_K>
 __device__ __forceinline__ void collide_pair(const Params<F2> &pw, float f[2][9], const float A3[2], const float A35[2],
                                              const float A5[2], float phi[2])
 {
@@ -111,7 +109,7 @@ __device__ __forceinline__ void collide_pair(const Params<F2> &pw, float f[2][9]
 #pragma unroll
     for (int k = 0; k < 9; ++k) g[k] = F2(f[0][k], f[1][k]);
     F2 ph;
-    collide<F2, CONV, DIFF, NODE_K>(pw, g, F2(A3[0], A3[1]), F2(A35[0], A35[1]), F2(A5[0], A5[1]), ph);
+    collide_stored<PREC, F2, CONV, DIFF, NODE_K>(pw, g, F2(A3[0], A3[1]), F2(A35[0], A35[1]), F2(A5[0], A5[1]), ph);
 #pragma unroll
     for (int k = 0; k < 9; ++k) { f[0][k] = g[k].v.x; f[1][k] = g[k].v.y; }
     phi[0] = ph.v.x;
@@ -163,10 +161,7 @@ __device__ __forceinline__ void step2_B(const Params<float> &p, const Params<F2>
                         const bool ox = p.abb_x && (xs < 0 || xs >= p.nx);
                         const bool oy = p.abb_y && (ys < 0 || ys >= p.ny);
                         if (ox || oy) {
-                            const float wx = xs < 0 ? p.phi_wall[0] : p.phi_wall[1];
-                            const float wy = ys < 0 ? p.phi_wall[2] : p.phi_wall[3];
-                            const float phiw = (ox && oy) ? 0.5f * (wx + wy) : (ox ? wx : wy);
-                            f[h][k] = wall_term<float, CONV, DIFF>(p, k, phiw) - sm[opp(k) * kRP + c];
+                            f[h][k] = wall_value<PREC, float, CONV, DIFF>(p, k, ox, oy) - sm[opp(k) * kRP + c];
                         }
                     }
                 }
@@ -182,7 +177,7 @@ __device__ __forceinline__ void step2_B(const Params<float> &p, const Params<F2>
                 A5[h] = __ldg(p.Afield + 2 * P + own[h]);
             }
         }
-        collide_pair<CONV, DIFF, KF>(pw, f, A3, A35, A5, phi);
+        collide_pair<PREC, CONV, DIFF, KF>(pw, f, A3, A35, A5, phi);
 #pragma unroll
         for (int h = 0; h < 2; ++h)
             if (ok[h]) S::store_cell(dst, dst_h, P, own[h], f[h], phi[h]);
@@ -242,7 +237,7 @@ __device__ __forceinline__ void two_steps(const Params<float> &p, const typename
                 A5[h] = __ldg(p.Afield + 2 * P + own);
             }
         }
-        collide_pair<CONV, DIFF, KF>(pw, f, A3, A35, A5, phi);
+        collide_pair<PREC, CONV, DIFF, KF>(pw, f, A3, A35, A5, phi);
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             if (INTERIOR || ok[h]) {

@@ -101,7 +101,7 @@ __device__ __forceinline__ void pull_row(const Params<float> &p, const typename 
 
 // anti-bounce-back for a wall node: links whose source lies outside take
 // -f*_opp(k)(own) + the even equilibrium part at the wall value
-template <int CONV, int DIFF, class OwnOpp>
+template <int PREC, int CONV, int DIFF, class OwnOpp>
 __device__ __forceinline__ void walls(const Params<float> &p, int x, int y, float f[9], OwnOpp own_opp)
 {
     const bool wall = (p.abb_x && (x == 0 || x == p.nx - 1)) || (p.abb_y && (y == 0 || y == p.ny - 1));
@@ -112,10 +112,7 @@ __device__ __forceinline__ void walls(const Params<float> &p, int x, int y, floa
         const bool ox = p.abb_x && (xs < 0 || xs >= p.nx);
         const bool oy = p.abb_y && (ys < 0 || ys >= p.ny);
         if (ox || oy) {
-            const float wx = xs < 0 ? p.phi_wall[0] : p.phi_wall[1];
-            const float wy = ys < 0 ? p.phi_wall[2] : p.phi_wall[3];
-            const float phiw = (ox && oy) ? 0.5f * (wx + wy) : (ox ? wx : wy);
-            f[k] = wall_term<float, CONV, DIFF>(p, k, phiw) - own_opp(opp(k));
+            f[k] = wall_value<PREC, float, CONV, DIFF>(p, k, ox, oy) - own_opp(opp(k));
         }
     }
 }
@@ -163,17 +160,17 @@ __device__ __forceinline__ void march(const Params<float> &p, const typename Sto
         float G[9];
         pull_row<PREC, CONV, DIFF, INTERIOR>(p, src, src_h, lane, xc, xl, xr, yrow, G);
         if (!INTERIOR && rowvalid && colvalid)
-            walls<CONV, DIFF>(p, xc, yrow, G, [&](int o) {
+            walls<PREC, CONV, DIFF>(p, xc, yrow, G, [&](int o) {
                 return Store<PREC>::ld(src + o * P, (long long)yrow * p.pitch + xc, src_h, wgt<float>(o));
             });
         {
             const long long own = (long long)yrow * p.pitch + xc;
             float phi;
             if (p.Afield)
-                collide<float, CONV, DIFF, true>(p, G, __ldg(p.Afield + own), __ldg(p.Afield + P + own),
+                collide_stored<PREC, float, CONV, DIFF, true>(p, G, __ldg(p.Afield + own), __ldg(p.Afield + P + own),
                                                  __ldg(p.Afield + 2 * P + own), phi);
             else
-                collide<float, CONV, DIFF, false>(p, G, p.A3, p.A35, p.A5, phi);
+                collide_stored<PREC, float, CONV, DIFF, false>(p, G, p.A3, p.A35, p.A5, phi);
         }
         // ---- step B: row yb = ya - 1 at time n+2 ------------------------------
         const int yb = ya - 1;
@@ -189,17 +186,17 @@ __device__ __forceinline__ void march(const Params<float> &p, const typename Sto
             f[7] = __shfl_down_sync(kFullM, G[7], 1);
             f[8] = __shfl_up_sync(kFullM, G[8], 1);
             if (out_lane) {
-                if (!INTERIOR) walls<CONV, DIFF>(p, xo, yb, f, [&](int o) { return P1[o]; });
+                if (!INTERIOR) walls<PREC, CONV, DIFF>(p, xo, yb, f, [&](int o) { return P1[o]; });
                 int xs = xo, ys = yb;
                 LBM_CHK(xs, p.nx, p.err, kErrX);
                 LBM_CHK(ys, p.ny, p.err, kErrY);
                 const long long own = (long long)ys * p.pitch + xs;
                 float phi;
                 if (p.Afield)
-                    collide<float, CONV, DIFF, true>(p, f, __ldg(p.Afield + own), __ldg(p.Afield + P + own),
+                    collide_stored<PREC, float, CONV, DIFF, true>(p, f, __ldg(p.Afield + own), __ldg(p.Afield + P + own),
                                                      __ldg(p.Afield + 2 * P + own), phi);
                 else
-                    collide<float, CONV, DIFF, false>(p, f, p.A3, p.A35, p.A5, phi);
+                    collide_stored<PREC, float, CONV, DIFF, false>(p, f, p.A3, p.A35, p.A5, phi);
                 S::store_cell(dst, dst_h, P, own, f, phi);
             }
         }

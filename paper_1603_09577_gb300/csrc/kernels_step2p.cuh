@@ -134,7 +134,7 @@ __device__ __forceinline__ void two_steps_pair(const Params<float> &p, const typ
     constexpr int kRY = TileP<TY>::kRY, kRP = TileP<TY>::kRP;
     constexpr int kWarps = kT2Threads / 32;
     const Params<F2> pw = widen(p);
-    const int lane = threadIdx.x, warp = threadIdx.y;
+    const int lane = threadIdx.x, warp = __shfl_sync(0xffffffffu, threadIdx.y, 0);
     const long long P = p.plane;
 
     // ---- step A: region row hy per warp pass, nodes (X0 - 1 + 2 lane, +1) ----
@@ -190,7 +190,7 @@ __device__ __forceinline__ void two_steps_pair(const Params<float> &p, const typ
             A35 = F2(__ldg(p.Afield + P + o0), __ldg(p.Afield + P + o1));
             A5 = F2(__ldg(p.Afield + 2 * P + o0), __ldg(p.Afield + 2 * P + o1));
         }
-        collide<F2, CONV, DIFF, KF>(pw, g, A3, A35, A5, ph);
+        collide_stored<PREC, F2, CONV, DIFF, KF>(pw, g, A3, A35, A5, ph);
         const int c = hy * kPRX + 2 * lane;
         if (INTERIOR || (ok[0] && ok[1])) {
 #pragma unroll
@@ -233,10 +233,7 @@ __device__ __forceinline__ void two_steps_pair(const Params<float> &p, const typ
                             const bool ox = p.abb_x && (xsrc < 0 || xsrc >= p.nx);
                             const bool oy = p.abb_y && (ysrc < 0 || ysrc >= p.ny);
                             if (ox || oy) {
-                                const float wx = xsrc < 0 ? p.phi_wall[0] : p.phi_wall[1];
-                                const float wy = ysrc < 0 ? p.phi_wall[2] : p.phi_wall[3];
-                                const float phiw = (ox && oy) ? 0.5f * (wx + wy) : (ox ? wx : wy);
-                                const float v = wall_term<float, CONV, DIFF>(p, k, phiw) - sm[opp(k) * kRP + c + h];
+                                const float v = wall_value<PREC, float, CONV, DIFF>(p, k, ox, oy) - sm[opp(k) * kRP + c + h];
                                 if (h == 0) g[k].v.x = v;
                                 else g[k].v.y = v;
                             }
@@ -255,7 +252,7 @@ __device__ __forceinline__ void two_steps_pair(const Params<float> &p, const typ
                 A35 = F2(__ldg(p.Afield + P + own), __ldg(p.Afield + P + o1));
                 A5 = F2(__ldg(p.Afield + 2 * P + own), __ldg(p.Afield + 2 * P + o1));
             }
-            collide<F2, CONV, DIFF, KF>(pw, g, A3, A35, A5, ph);
+            collide_stored<PREC, F2, CONV, DIFF, KF>(pw, g, A3, A35, A5, ph);
             store_pair<PREC>(p, dst, dst_h, own, g, ph, both);
         }
     }
@@ -316,13 +313,13 @@ static cudaError_t step2p_ty(const lbm_solver *s, int src, cudaStream_t st)
     return cudaGetLastError();
 }
 
-// tile height from the descriptor: block_rows 4 selects 62 x 14 tiles (37 KB of
-// shared memory, 4 blocks per SM), 2 selects 62 x 22 (55 KB, 4 blocks), anything
-// else 62 x 30 (74 KB, 3 blocks)
+// tile height from the descriptor: block_rows 4, or an automatic choice, selects
+// 62 x 14 tiles (37 KB of shared memory, 4 blocks per SM), 2 selects 62 x 22 (55 KB,
+// 4 blocks), anything else 62 x 30 (74 KB, 3 blocks)
 template <int PREC, int CONV, int DIFF, bool KF>
 static cudaError_t step2p_k(const lbm_solver *s, int src, cudaStream_t st)
 {
-    if (s->d.block_rows == 4) return step2p_ty<PREC, CONV, DIFF, 14, KF>(s, src, st);
+    if (s->d.block_rows == 4 || s->d.kernel_variant == 0) return step2p_ty<PREC, CONV, DIFF, 14, KF>(s, src, st);
     if (s->d.block_rows == 2) return step2p_ty<PREC, CONV, DIFF, 22, KF>(s, src, st);
     return step2p_ty<PREC, CONV, DIFF, 30, KF>(s, src, st);
 }

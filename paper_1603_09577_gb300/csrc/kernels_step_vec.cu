@@ -201,10 +201,7 @@ k_step_v4(const Params<float> p, const typename VecIO<PREC>::T *__restrict__ src
                 const bool ox = p.abb_x && (xs < 0 || xs >= p.nx);
                 const bool oy = p.abb_y && (ys < 0 || ys >= p.ny);
                 if (ox || oy) {
-                    const float wx = xs < 0 ? p.phi_wall[0] : p.phi_wall[1];
-                    const float wy = ys < 0 ? p.phi_wall[2] : p.phi_wall[3];
-                    const float phiw = (ox && oy) ? 0.5f * (wx + wy) : (ox ? wx : wy);
-                    f[c][k] = wall_term<float, CONV, DIFF>(p, k, phiw) -
+                    f[c][k] = wall_value<PREC, float, CONV, DIFF>(p, k, ox, oy) -
                               S::ld(src + opp(k) * P, own, src_h, wgt<float>(opp(k)));
                 }
             }
@@ -231,10 +228,10 @@ k_step_v4(const Params<float> p, const typename VecIO<PREC>::T *__restrict__ src
     float phi[4];
     if (p.Afield) {
 #pragma unroll
-        for (int c = 0; c < 4; ++c) collide<float, CONV, DIFF, true>(p, f[c], A3[c], A35[c], A5[c], phi[c]);
+        for (int c = 0; c < 4; ++c) collide_stored<PREC, float, CONV, DIFF, true>(p, f[c], A3[c], A35[c], A5[c], phi[c]);
     } else {
 #pragma unroll
-        for (int c = 0; c < 4; ++c) collide<float, CONV, DIFF, false>(p, f[c], A3[c], A35[c], A5[c], phi[c]);
+        for (int c = 0; c < 4; ++c) collide_stored<PREC, float, CONV, DIFF, false>(p, f[c], A3[c], A35[c], A5[c], phi[c]);
     }
     if (active) IO::store(dst, dst_h, P, r0 + L.x0, f, phi);
 }

@@ -131,6 +131,26 @@ static bool relax_block(const double K[3], double *A3, double *A35, double *A5)
     return true;
 }
 
+// feq_k + feq_opp(k) (Eq. 3, its even part) at the wall values, per direction and
+// crossed walls, for the families the table serves (conv 0 and 1, diff 0 to 2)
+template <class C>
+static void wall_table(const lbm_solver *s, C wt[8][3])
+{
+    const lbm_coeffs &c = s->c;
+    for (int k = 1; k < 9; ++k)
+        for (int z = 0; z < 3; ++z) {
+            const double wx = s->d.phi_wall[cx(k) > 0 ? 0 : 1], wy = s->d.phi_wall[cy(k) > 0 ? 2 : 3];
+            const double phi = z == 0 ? wx : (z == 1 ? wy : 0.5 * (wx + wy));
+            const double cphi = c.conv == 0 ? phi : phi * phi * phi / 3.0;
+            const double g = c.diff == 0 ? phi : (c.diff == 1 ? phi + 0.5 * phi * phi : phi + phi * phi * phi / 3.0);
+            const double Qxx = c.u[0] * c.u[0] * cphi + (g - phi) / 3.0, Qyy = c.u[1] * c.u[1] * cphi + (g - phi) / 3.0;
+            const double Qxy = c.u[0] * c.u[1] * cphi;
+            const double qc = Qxx * (cx(k) * cx(k) - 1.0 / 3.0) + 2.0 * cx(k) * cy(k) * Qxy +
+                              Qyy * (cy(k) * cy(k) - 1.0 / 3.0);
+            wt[k - 1][z] = (C)(2.0 * wgt<double>(k) * (phi + 4.5 * qc));
+        }
+}
+
 template <class C>
 Params<C> make_params(const lbm_solver *s)
 {
@@ -173,6 +193,8 @@ Params<C> make_params(const lbm_solver *s)
     p.nee_y = s->d.bc_y == LBM_NEE;
     p.bv = nullptr;
     if (p.fisher) p.has_src = 1;
+    p.k = coll_cast<C>(make_coll(c, A3, A35, A5));
+    wall_table<C>(s, p.wt);
     return p;
 }
 

@@ -24,10 +24,10 @@ __host__ __device__ constexpr C wgt(int k) { return k == 0 ? C(4) / C(9) : (k <=
 // packed add / multiply / fused multiply-add for both (sm_100 and later).
 struct F2 {
     float2 v;
-    __device__ __forceinline__ F2() {}
-    __device__ __forceinline__ F2(float s) : v(make_float2(s, s)) {}
-    __device__ __forceinline__ F2(float a, float b) : v(make_float2(a, b)) {}
-    __device__ __forceinline__ explicit F2(float2 a) : v(a) {}
+    __host__ __device__ __forceinline__ F2() {}
+    __host__ __device__ __forceinline__ F2(float s) : v(make_float2(s, s)) {}
+    __host__ __device__ __forceinline__ F2(float a, float b) : v(make_float2(a, b)) {}
+    __host__ __device__ __forceinline__ explicit F2(float2 a) : v(a) {}
 };
 __device__ __forceinline__ F2 operator+(F2 a, F2 b) { return F2(__fadd2_rn(a.v, b.v)); }
 __device__ __forceinline__ F2 operator*(F2 a, F2 b) { return F2(__fmul2_rn(a.v, b.v)); }
@@ -39,6 +39,41 @@ __device__ __forceinline__ F2 &operator-=(F2 &a, F2 b) { a = a - b; return a; }
 // a * b + c: fused for the packed type, left to contraction for scalars
 template <class C> __device__ __forceinline__ C mad(C a, C b, C c) { return a * b + c; }
 template <> __device__ __forceinline__ F2 mad<F2>(F2 a, F2 b, F2 c) { return F2(__ffma2_rn(a.v, b.v, c.v)); }
+
+// ---- constants of the collision relax() (lbm_relax.cuh) ------------------------
+// Rates, equilibrium polynomials, source factors and the constant relaxation
+// block, each computed in double on the host and rounded once. All members have
+// the type C (coll_cast converts them as an array).
+template <class C>
+struct Coll {
+    C nse1, nse2;               // -s1/36, -s2/36
+    C sq4, nsq4, sq6, nsq6;     // s4/6, -s4/12, s6/6, -s6/12
+    C sp7, nsp7, sp8, nsp8;     // +/- s7/4, +/- s8/4
+    C na3, na35, na5;           // -A3/6, -A35/6, -A5/6 (Eq. 17, 26)
+    C ke1, nkp1, ke3;           // e_eq = ke1 phi + h, eps_eq = kp1 phi - h, h = [phi^2] + ke3 phi^3
+    C bx, by, nbx, nby;         // B = b beta (beta = phi, or phi^2 with b = a/2), and -b
+    C nkxx, nkxy;               // -(C_xx - C_yy), -C_xy per phi (conv 0) or phi^3 (conv 1)
+    C inv_den, phi0;            // Eq. 35: phi = inv_den rho + phi0
+    C r0, r1, ninth;            // R = r0 + r1 phi; 1/9
+    C nhe1, he2;                // source factors of -e and eps
+    C hqx, hqy, hqx2, hqy2;     // of q_x, q_y, and of -2 q_x, -2 q_y
+    C jsx, jsy;                 // (I - A/2) B' / 6 of the constant block
+    C ux, uy, sixth, nsixth;    // B' = u (conv 0) or u phi; 1/6, -1/6
+    C four, mtwo, half;         // 4, -2, 1/2
+};
+
+template <class D, class S>
+__host__ __device__ __forceinline__ Coll<D> coll_cast(const Coll<S> &a)
+{
+    Coll<D> r;
+    constexpr int n = sizeof(Coll<S>) / sizeof(S);
+    static_assert(sizeof(Coll<D>) == n * sizeof(D), "all members of Coll have its type");
+    const S *s = reinterpret_cast<const S *>(&a);
+    D *d = reinterpret_cast<D *>(&r);
+#pragma unroll
+    for (int i = 0; i < n; ++i) d[i] = D(s[i]);
+    return r;
+}
 
 // ---- kernel parameters (passed by value) -----------------------------------
 // Relaxation rates, flux and source coefficients in the compute type C.
@@ -73,6 +108,10 @@ struct Params {
     C b;
     int nee_x, nee_y;       // 1: non-equilibrium extrapolation on that axis
     const double *bv;       // Dirichlet record of this step: west, east, south, north
+    Coll<C> k;              // constants of relax()
+    // anti-bounce-back: feq_k + feq_opp(k) at the wall value of direction k = 1..8
+    // when its link crosses an x wall, a y wall, both (mean value)
+    C wt[8][3];
 };
 
 // ---- checked builds ------------------------------------------------------------

@@ -9,7 +9,7 @@
 #include <string>
 
 #include "lbm.h"
-#include "lbm_device.cuh"
+#include "lbm_relax.cuh"
 
 namespace lbm {
 
@@ -45,6 +45,7 @@ struct lbm_solver {
     double *check = nullptr;        // 8 doubles: reduction output of lbm_check_finite
     int *err = nullptr;             // index-fault word of checked builds
     int cur = 0;
+    int sms = 0;                    // SMs of the device, read at the first step
     long long t = 0;
     // Dirichlet records of the extrapolated axes (caller-owned device memory)
     const double *dir_vals = nullptr;
@@ -105,6 +106,39 @@ inline void set_scaled_rates(const double s[9], double A3, double A35, double A5
     p->c3s = (C)(1.0 / 6.0 - A3 / 12.0); p->c35s = (C)(-A35 / 12.0); p->c5s = (C)(1.0 / 6.0 - A5 / 12.0);
 }
 
+// the constants of relax() for the coefficients c and the block A
+inline Coll<double> make_coll(const lbm_coeffs &c, double A3, double A35, double A5)
+{
+    Coll<double> k;
+    const double *s = c.s;
+    const double ux = c.u[0], uy = c.u[1], uu = ux * ux + uy * uy;
+    const double h1 = 1.0 - 0.5 * s[1], h2 = 1.0 - 0.5 * s[2], h4 = 1.0 - 0.5 * s[4], h6 = 1.0 - 0.5 * s[6];
+    const bool quad = c.conv == 1;                    // B = a phi^2/2, C = a a phi^3/3
+    k.nse1 = -s[1] / 36.0; k.nse2 = -s[2] / 36.0;
+    k.sq4 = s[4] / 6.0; k.nsq4 = -s[4] / 12.0; k.sq6 = s[6] / 6.0; k.nsq6 = -s[6] / 12.0;
+    k.sp7 = s[7] / 4.0; k.nsp7 = -k.sp7; k.sp8 = s[8] / 4.0; k.nsp8 = -k.sp8;
+    k.na3 = -A3 / 6.0; k.na35 = -A35 / 6.0; k.na5 = -A5 / 6.0;
+    k.ke1 = quad ? -2.0 : 3.0 * uu - 2.0;
+    k.nkp1 = quad ? -1.0 : 3.0 * uu - 1.0;
+    k.ke3 = (quad ? uu : 0.0) + (c.diff == 2 ? 2.0 / 3.0 : 0.0);
+    const double half = quad ? 0.5 : 1.0, third = quad ? 1.0 / 3.0 : 1.0;
+    k.bx = half * ux; k.by = half * uy;
+    k.nbx = -k.bx; k.nby = -k.by;
+    k.nkxx = -third * (ux * ux - uy * uy);
+    k.nkxy = -third * ux * uy;
+    k.inv_den = 1.0 / (1.0 - 0.5 * c.r1);
+    k.phi0 = 0.5 * c.r0 * k.inv_den;
+    k.r0 = c.r0; k.r1 = c.r1; k.ninth = 1.0 / 9.0;
+    k.nhe1 = 2.0 * h1 / 36.0; k.he2 = h2 / 36.0;
+    k.hqx = -h4 / 12.0 * ux; k.hqy = -h6 / 12.0 * uy;
+    k.hqx2 = h4 / 6.0 * ux; k.hqy2 = h6 / 6.0 * uy;
+    k.jsx = (1.0 / 6.0 - A3 / 12.0) * ux - A35 / 12.0 * uy;
+    k.jsy = -A35 / 12.0 * ux + (1.0 / 6.0 - A5 / 12.0) * uy;
+    k.ux = ux; k.uy = uy; k.sixth = 1.0 / 6.0; k.nsixth = -1.0 / 6.0;
+    k.four = 4.0; k.mtwo = -2.0; k.half = 0.5;
+    return k;
+}
+
 cudaError_t launch_init(const lbm_solver *s, const void *phi, int in_prec, cudaStream_t st);
 cudaError_t launch_step(const lbm_solver *s, int src, cudaStream_t st);
 cudaError_t launch_step2(const lbm_solver *s, int src, cudaStream_t st);
@@ -124,6 +158,11 @@ cudaError_t launch_general_f32(const lbm_solver *s, int src, const double *bv, c
 cudaError_t launch_step2_general(const lbm_solver *s, int src, const double *records, cudaStream_t st);
 // advance the device record count by `by` steps (one thread, after a call's sweeps)
 cudaError_t launch_tick(long long *counter, int by, cudaStream_t st);
+// four steps per sweep of an FP32 lattice (kernels_march.cuh); prepare: only the
+// kernel's attributes, so that a later first launch may happen under capture
+cudaError_t launch_march_src(const lbm_solver *s, int src, bool prepare, cudaStream_t st);
+cudaError_t launch_march_free(const lbm_solver *s, int src, bool prepare, cudaStream_t st);
+cudaError_t launch_march_kfield(const lbm_solver *s, int src, bool prepare, cudaStream_t st);
 bool step_v4_supported(const lbm_solver *s);
 bool step_v4_preferred(const lbm_solver *s);
 cudaError_t launch_step_v4(const lbm_solver *s, int src, cudaStream_t st);
