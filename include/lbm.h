@@ -78,9 +78,16 @@ typedef struct {
     int bc_x, bc_y;         /* LBM_PERIODIC, LBM_ABB or LBM_NEE per axis          */
     double phi_wall[4];     /* Dirichlet values: west, east, south, north         */
     int steps_per_pass;     /* 1, or 2: two time steps per sweep through memory
-                               (F32 and BF16S with periodic or ABB walls)         */
+                               (F32 and BF16S with periodic or ABB walls). LBM_F32
+                               with an automatic launch (below) may take more steps
+                               per sweep in either case: the populations are the
+                               same bit for bit, and a call's launches stay even or
+                               odd in number as without it                        */
     int per_cell_K;         /* 1: K comes from lbm_set_K_field                    */
-    int kernel_variant;     /* 0: automatic; 1: one node per thread; 2: four
+    int kernel_variant;     /* 0: automatic (LBM_F32 with block_rows 0, Scheme B,
+                               conv 0 / 1, diff 0 to 2: the library chooses the
+                               steps per sweep by the lattice's size); 1: one node
+                               per thread; 2: four
                                x-adjacent nodes per thread with vector loads
                                (LBM_F32 / LBM_BF16S, nx % 4 == 0); 3: with
                                steps_per_pass 2, the register column march (each
@@ -90,7 +97,8 @@ typedef struct {
                                tile's input staged by a TMA tensor copy; 5: with
                                steps_per_pass 2 (LBM_F32 / LBM_BF16S), the tile
                                kernel with two x-adjacent nodes per thread and
-                               paired (vector) loads and stores               */
+                               paired (vector) loads and stores; with block_rows
+                               4 and LBM_F32 as 0, automatic                  */
     int block_rows;         /* rows of 32-thread warps per thread block: 0 (= 8),
                                1, 2, 4 or 8; for kernel_variant 3 the rows each
                                warp marches are 16 * block_rows (0: 64); for the
@@ -170,7 +178,8 @@ int lbm_set_phi(lbm_handle h, const void *dev_phi, int prec, void *stream);
    boundaries of lbm_desc). Asynchronous; no host synchronisation. The kernels
    alternate between the two population buffers; a stream capture of an even
    number of launches (nsteps even, or with steps_per_pass 2 a multiple of 4)
-   therefore replays consistently. The first call on a device configures kernel
+   therefore replays consistently. (Sweeps of more than two steps keep that: their
+   number is chosen so that the launches of a call are even or odd as before.) The first call on a device configures kernel
    attributes: make it before any stream capture. */
 int lbm_step(lbm_handle h, int nsteps, void *stream);
 
@@ -218,7 +227,7 @@ int lbm_check_finite(lbm_handle h, long long *nonfinite, void *stream);
    lbm_set_phi), synchronising `stream`; lbm_build_checked returns 1 in a checked
    build, 0 otherwise. In every build, a BF16S pair-tile launch (kernel_variant 5)
    whose grid would not cover the lattice writes nothing and sets 32, and the
-   TMA-staged kernel's bounded wait sets 16 (below); otherwise the word stays 0
+   bounded waits of the kernels that stage their input by bulk copies set 16 (below); otherwise the word stays 0
    in normal builds. */
 int lbm_debug_flags(lbm_handle h, int *flags, void *stream);
 int lbm_build_checked(void);

@@ -216,6 +216,77 @@ static cudaError_t launch_general(const lbm_solver *s, int src, const double *bv
     return cudaErrorInvalidValue;
 }
 
+// FP32 lattices of Scheme B whose launch is left to the library: kernel_variant 0
+// without a block shape, or the pair kernels' small tiles (kernel_variant 5,
+// block_rows 4). The kernels agree bit for bit, whatever the split into sweeps; with
+// a per-node tensor the one-step kernel differs in the last bit from the others, so
+// that one step per pass there stays one step.
+static bool auto_path(const lbm_solver *s)
+{
+    return s->d.prec == LBM_F32 && !(s->d.per_cell_K && s->d.steps_per_pass == 1) && ((s->d.kernel_variant == 0 && s->d.block_rows == 0) ||
+                                    (s->d.kernel_variant == 5 && s->d.block_rows == 4));
+}
+
+// Whether sweeps of four steps by the marching kernel serve this lattice. They need
+// strips and chunks for the whole chip: from about 2^18 nodes on.
+static bool march_wanted(const lbm_solver *s)
+{
+    return s->d.nx >= 128 && s->d.ny >= 64 && (long long)s->d.nx * s->d.ny >= (1LL << 18) && s->L.plane < (1LL << 31);
+}
+
+static cudaError_t launch_march(const lbm_solver *s, int src, bool prepare, cudaStream_t st)
+{
+    if (s->d.per_cell_K) return launch_march_kfield(s, src, prepare, st);
+    if (s->c.r0 != 0.0 || s->c.r1 != 0.0) return launch_march_src(s, src, prepare, st);
+    return launch_march_free(s, src, prepare, st);
+}
+
+static int device_sms(lbm_solver *s)
+{
+    if (s->sms > 0) return LBM_OK;
+    int dev = 0;
+    if (int rc = cuda_check(cudaGetDevice(&dev), "cudaGetDevice")) return rc;
+    return cuda_check(cudaDeviceGetAttribute(&s->sms, cudaDevAttrMultiProcessorCount, dev), "SM count");
+}
+
+// nsteps as sweeps of four, two and one steps. The number of launches stays odd or
+// even as it is with steps_per_pass steps each (n, or n/2 + n%2), so that a
+// captured call that ended on the buffer it started from still does: with m pairs
+// of steps, sweeps of four are even in number (two steps per pass) or as m (one).
+static int step_auto(lbm_handle h, int nsteps, cudaStream_t st)
+{
+    if (int rc = device_sms(h)) return rc;
+    const int m = nsteps / 2, one = nsteps % 2;
+    int four = 0;
+    if (march_wanted(h)) {
+        if (int rc = cuda_check(launch_march(h, h->cur, true, st), "lbm_step (kernel attributes)")) return rc;
+        four = m / 2;
+        if ((four & 1) != (h->d.steps_per_pass == 2 ? 0 : (m & 1))) --four;
+        if (four < 0) four = 0;
+    }
+    int two = m - 2 * four, single = one;
+    if (h->d.steps_per_pass == 1 && ((four + two) & 1)) {     // no sweeps of four to make the count even
+        --two;
+        single += 2;
+    }
+    for (int i = 0; i < four; ++i) {
+        if (int rc = cuda_check(launch_march(h, h->cur, false, st), "lbm_step (four steps per sweep)")) return rc;
+        h->cur ^= 1;
+        h->t += 4;
+    }
+    for (int i = 0; i < two; ++i) {
+        if (int rc = cuda_check(launch_step2p_f32(h, h->cur, st), "lbm_step (two steps per sweep)")) return rc;
+        h->cur ^= 1;
+        h->t += 2;
+    }
+    for (int i = 0; i < single; ++i) {
+        if (int rc = cuda_check(launch_step(h, h->cur, st), "lbm_step")) return rc;
+        h->cur ^= 1;
+        h->t += 1;
+    }
+    return LBM_OK;
+}
+
 static int check_handle(lbm_handle h)
 {
     if (!h) return fail(LBM_EINVAL, "null handle");
@@ -443,6 +514,7 @@ int lbm_step(lbm_handle h, int nsteps, void *stream)
             if (int rc = cuda_check(launch_tick(h->dir_counter, nsteps, st), "lbm_step (records)")) return rc;
         return LBM_OK;
     }
+    if (auto_path(h)) return step_auto(h, nsteps, st);
     if (h->d.steps_per_pass == 2) {
         for (; done + 2 <= nsteps; done += 2) {
             const cudaError_t e = h->d.kernel_variant == 3   ? launch_step2m(h, h->cur, st)
