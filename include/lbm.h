@@ -79,14 +79,14 @@ typedef struct {
     double phi_wall[4];     /* Dirichlet values: west, east, south, north         */
     int steps_per_pass;     /* 1, or 2: two time steps per sweep through memory
                                (F32 and BF16S with periodic or ABB walls). LBM_F32
-                               with an automatic launch (below) may take more steps
-                               per sweep in either case: the populations are the
+                               and LBM_F64 with an automatic launch (below) may take
+                               more steps per sweep in either case: the populations are the
                                same bit for bit, and a call's launches stay even or
                                odd in number as without it                        */
     int per_cell_K;         /* 1: K comes from lbm_set_K_field                    */
-    int kernel_variant;     /* 0: automatic (LBM_F32 with block_rows 0, Scheme B,
-                               conv 0 / 1, diff 0 to 2: the library chooses the
-                               steps per sweep by the lattice's size); 1: one node
+    int kernel_variant;     /* 0: automatic (LBM_F32 and LBM_F64 with block_rows 0,
+                               Scheme B, conv 0 / 1, diff 0 to 2: the library
+                               chooses the steps per sweep by the lattice's size); 1: one node
                                per thread; 2: four
                                x-adjacent nodes per thread with vector loads
                                (LBM_F32 / LBM_BF16S, nx % 4 == 0); 3: with

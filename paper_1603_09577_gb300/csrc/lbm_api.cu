@@ -6,6 +6,7 @@
 #include <stdio.h>
 #include <string.h>
 
+#include <algorithm>
 #include <new>
 #include <string>
 
@@ -216,15 +217,40 @@ static cudaError_t launch_general(const lbm_solver *s, int src, const double *bv
     return cudaErrorInvalidValue;
 }
 
-// FP32 lattices of Scheme B whose launch is left to the library: kernel_variant 0
-// without a block shape, or the pair kernels' small tiles (kernel_variant 5,
-// block_rows 4). The kernels agree bit for bit, whatever the split into sweeps; with
-// a per-node tensor the one-step kernel differs in the last bit from the others, so
-// that one step per pass there stays one step.
+// Lattices of Scheme B whose launch is left to the library: FP64 and FP32 with
+// kernel_variant 0 and no block shape, or FP32 with the pair kernels' small tiles
+// (kernel_variant 5, block_rows 4). The kernels of a precision agree bit for bit,
+// whatever the split into sweeps; only with a per-node tensor in FP32 does the
+// one-step kernel differ in the last bit, so that one step per pass stays one there.
 static bool auto_path(const lbm_solver *s)
 {
-    return s->d.prec == LBM_F32 && !(s->d.per_cell_K && s->d.steps_per_pass == 1) && ((s->d.kernel_variant == 0 && s->d.block_rows == 0) ||
-                                    (s->d.kernel_variant == 5 && s->d.block_rows == 4));
+    if (s->d.prec == LBM_F64) return s->d.kernel_variant == 0 && s->d.block_rows == 0;
+    return s->d.prec == LBM_F32 && !(s->d.per_cell_K && s->d.steps_per_pass == 1) &&
+           ((s->d.kernel_variant == 0 && s->d.block_rows == 0) || (s->d.kernel_variant == 5 && s->d.block_rows == 4));
+}
+
+static cudaError_t launch_tile(const lbm_solver *s, int src, int steps, bool prepare, cudaStream_t st)
+{
+    if (s->d.prec == LBM_F64)
+        return s->d.per_cell_K ? launch_tile_f64_kfield(s, src, steps, prepare, st)
+                               : launch_tile_f64_const(s, src, steps, prepare, st);
+    return s->d.per_cell_K ? launch_tile_f32_kfield(s, src, steps, prepare, st)
+                           : launch_tile_f32_const(s, src, steps, prepare, st);
+}
+
+// Whether the tiles of s->plan are estimated faster per step than the large
+// lattices' kernels (microseconds). FP32, the marching kernel and the pair tiles:
+// 4.14 at 400^2 (tiles 2.18), 4.17 at 600^2 (4.00), 5.74 at 803 x 797 (7.00). FP64, the
+// one-step kernel, whose blocks of 256 nodes take two turns of an SM's FP64 pipe
+// each: 8.28 at 128^2 (tiles 5.21), 14.4 at 200^2 (9.31), 19.0 at 301^2 (16.9).
+static bool tile_wanted(const lbm_solver *s)
+{
+    const double n = (double)s->d.nx * s->d.ny;
+    if (s->d.prec == LBM_F64) {
+        const long long blocks = (long long)((s->d.nx + 31) / 32) * ((s->d.ny + 7) / 8);
+        return s->plan.us < 3.2 + 5.2 * (double)((blocks + s->sms - 1) / s->sms);
+    }
+    return s->plan.us < std::max(4.1, 2.5 + n / 210e3);
 }
 
 // Whether sweeps of four steps by the marching kernel serve this lattice. They need
@@ -256,9 +282,25 @@ static int device_sms(lbm_solver *s)
 static int step_auto(lbm_handle h, int nsteps, cudaStream_t st)
 {
     if (int rc = device_sms(h)) return rc;
-    const int m = nsteps / 2, one = nsteps % 2;
+    if (h->plan.T == 0) h->plan = tile_plan(h->d.nx, h->d.ny, h->d.prec == LBM_F64, h->sms);
+    if (tile_wanted(h)) {
+        if (int rc = cuda_check(launch_tile(h, h->cur, 1, true, st), "lbm_step (kernel attributes)")) return rc;
+        // as few launches as hold nsteps, even or odd in number as promised, of nearly equal size
+        const int wanted = h->d.steps_per_pass == 2 ? nsteps / 2 + nsteps % 2 : nsteps;
+        int launches = (nsteps + h->plan.T - 1) / h->plan.T;
+        if (((launches ^ wanted) & 1) && launches < nsteps) ++launches;
+        for (int i = 0, done = 0; i < launches; ++i) {
+            const int steps = (nsteps - done) / (launches - i) + ((nsteps - done) % (launches - i) != 0);
+            if (int rc = cuda_check(launch_tile(h, h->cur, steps, false, st), "lbm_step (small lattice)")) return rc;
+            h->cur ^= 1;
+            h->t += steps;
+            done += steps;
+        }
+        return LBM_OK;
+    }
+    const int m = h->d.prec == LBM_F64 ? 0 : nsteps / 2, one = nsteps - 2 * m;
     int four = 0;
-    if (march_wanted(h)) {
+    if (h->d.prec == LBM_F32 && march_wanted(h)) {
         if (int rc = cuda_check(launch_march(h, h->cur, true, st), "lbm_step (kernel attributes)")) return rc;
         four = m / 2;
         if ((four & 1) != (h->d.steps_per_pass == 2 ? 0 : (m & 1))) --four;

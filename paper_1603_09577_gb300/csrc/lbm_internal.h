@@ -29,6 +29,17 @@ int make_layout(const lbm_desc *d, Layout *L);
 
 }  // namespace lbm
 
+namespace lbm {
+
+// Launch of a small lattice: W x H tiles, T steps per launch (kernels_tile.cuh); us:
+// the estimated time of a step. T = 0: not planned yet.
+struct TilePlan {
+    int W, H, T;
+    double us;
+};
+
+}  // namespace lbm
+
 struct lbm_solver {
     lbm_desc d;
     lbm_coeffs c;
@@ -46,6 +57,7 @@ struct lbm_solver {
     int *err = nullptr;             // index-fault word of checked builds
     int cur = 0;
     int sms = 0;                    // SMs of the device, read at the first step
+    lbm::TilePlan plan{0, 0, 0, 0.0};
     long long t = 0;
     // Dirichlet records of the extrapolated axes (caller-owned device memory)
     const double *dir_vals = nullptr;
@@ -163,6 +175,12 @@ cudaError_t launch_tick(long long *counter, int by, cudaStream_t st);
 cudaError_t launch_march_src(const lbm_solver *s, int src, bool prepare, cudaStream_t st);
 cudaError_t launch_march_free(const lbm_solver *s, int src, bool prepare, cudaStream_t st);
 cudaError_t launch_march_kfield(const lbm_solver *s, int src, bool prepare, cudaStream_t st);
+// `steps` steps in one launch over the tiles of s->plan (kernels_tile.cuh)
+TilePlan tile_plan(int nx, int ny, bool f64, int sms);
+cudaError_t launch_tile_f32_const(const lbm_solver *s, int src, int steps, bool prepare, cudaStream_t st);
+cudaError_t launch_tile_f32_kfield(const lbm_solver *s, int src, int steps, bool prepare, cudaStream_t st);
+cudaError_t launch_tile_f64_const(const lbm_solver *s, int src, int steps, bool prepare, cudaStream_t st);
+cudaError_t launch_tile_f64_kfield(const lbm_solver *s, int src, int steps, bool prepare, cudaStream_t st);
 bool step_v4_supported(const lbm_solver *s);
 bool step_v4_preferred(const lbm_solver *s);
 cudaError_t launch_step_v4(const lbm_solver *s, int src, cudaStream_t st);
