@@ -81,8 +81,10 @@ int lbm3_set_coeffs(lbm3_handle h, const lbm3_coeffs *c);
    collision). dev_phi: nx*ny*nz values of `prec` (LBM_F64 or LBM_F32). */
 int lbm3_set_phi(lbm3_handle h, const void *dev_phi, int prec, void *stream);
 /* Advance nsteps fused pull-stream / collide steps (asynchronous). The kernels
-   alternate between the two population buffers and need no function
-   attributes, so a stream capture of an even nsteps replays consistently. */
+   alternate between the two population buffers; a stream capture of an even
+   nsteps replays consistently. Large periodic LBM_F32 lattices with block_rows 0
+   take an even number of sweeps of two steps (the same states bit for bit); their
+   kernel's attributes are set by lbm3_set_phi, lbm3_load or the first call. */
 int lbm3_step(lbm3_handle h, int nsteps, void *stream);
 /* Checkpoint / resume: the state is lbm3_state_bytes bytes (the 19 population
    planes and, for LBM_BF16S, the shift plane). dev_dst / dev_src: device

@@ -118,6 +118,34 @@ __device__ __forceinline__ void store3(const Planes3<typename St3<PREC>::T> &pl,
     }
 }
 
+// constants of relax3() (lbm3_relax.cuh), computed in double on the host; all
+// members have the type C
+template <class C>
+struct Coll3 {
+    C omse;                     // 1 - s_e
+    C nb[3], ph[3];             // -B per beta (beta = phi, or phi^2 for conv 1), u/2
+    C nG[6];                    // -(A - s_e I)/10: xx, xy, xz, yy, yz, zz
+    C u6[3], u12[3];            // u/6, u/12
+    C tb, hse;                  // t = s_e B + (1 - s_e/2) R B' = u (tb beta + hse S)
+    C xs, xc, xi;               // X = xs phi + xc cphi + xi iso + hse R (cphi, iso: powers of phi)
+    C i18, i36, i3, qi;         // 1/18, 1/36, 1/3; s_e/4 times the isotropic part
+    C ea[3], ep[3], em[3];      // even parts per cphi (Params3)
+    C inv_den, phi0, r0, r1;
+};
+
+template <class D, class S>
+__host__ __device__ __forceinline__ Coll3<D> coll3_cast(const Coll3<S> &a)
+{
+    Coll3<D> r;
+    constexpr int n = sizeof(Coll3<S>) / sizeof(S);
+    static_assert(sizeof(Coll3<D>) == n * sizeof(D), "all members of Coll3 have its type");
+    const S *s = reinterpret_cast<const S *>(&a);
+    D *d = reinterpret_cast<D *>(&r);
+#pragma unroll
+    for (int i = 0; i < n; ++i) d[i] = D(s[i]);
+    return r;
+}
+
 template <class C>
 struct Params3 {
     int nx, ny, nz;
@@ -137,6 +165,10 @@ struct Params3 {
     int any_abb;
     C phi_wall[6];                   // x-, x+, y-, y+, z-, z+
     int *err;                        // checked builds: index-fault word
+    Coll3<C> k;
+    // feq_k + feq_opp(k) at the wall of direction k = 1..18, by the set of axes whose
+    // walls its link crosses (bit a: axis a; the mean value of the walls)
+    C wt[18][7];
 };
 
 // Coefficients at phi (Eq. 7 families, D = g(phi) I): B, B', the tensor
@@ -359,7 +391,16 @@ __device__ __forceinline__ void pull3_node(const Params3<typename St3<PREC>::C> 
                 if (p.abb[0] && (xs < 0 || xs >= p.nx)) { tot += xs < 0 ? p.phi_wall[0] : p.phi_wall[1]; ++cnt; }
                 if (p.abb[1] && (ys < 0 || ys >= p.ny)) { tot += ys < 0 ? p.phi_wall[2] : p.phi_wall[3]; ++cnt; }
                 if (p.abb[2] && (zs < 0 || zs >= p.nz)) { tot += zs < 0 ? p.phi_wall[4] : p.phi_wall[5]; ++cnt; }
-                if (cnt) {
+                if (PREC == LBM_F32) {
+                    const int set = (p.abb[0] && (xs < 0 || xs >= p.nx) ? 1 : 0) |
+                                    (p.abb[1] && (ys < 0 || ys >= p.ny) ? 2 : 0) |
+                                    (p.abb[2] && (zs < 0 || zs >= p.nz) ? 4 : 0);
+                    if (set) {
+                        const T back = OFF32 ? S::ld(pl.src0, own + pl.poff[opp3(k)], pl.src_h, own, w3<T>(opp3(k)))
+                                             : S::ld(pl.src[opp3(k)], own, pl.src_h, own, w3<T>(opp3(k)));
+                        f[k] = vsub(p.wt[k - 1][set - 1], back);
+                    }
+                } else if (cnt) {
                     const T phiw = cnt == 1 ? tot : tot / T(cnt);
                     const Coef3<CONV, DIFF, T> q(p, phiw);
                     const T back = OFF32 ? S::ld(pl.src0, own + pl.poff[opp3(k)], pl.src_h, own, w3<T>(opp3(k)))
