@@ -321,7 +321,10 @@ int lbm_ensemble_info(lbm_ensemble e, long long *nodes, int *tiles, int *grid);
 int lbm_ensemble_set_phi(lbm_ensemble e, const void *dev_phi, int prec, void *stream);
 /* Persistent launches advance 1 (default) or 2 time steps each; with 2, every
    launch runs a two-step shared-memory tile routine on the tiles of all
-   instances (two steps per sweep through HBM). Set before capturing a graph. */
+   instances (two steps per sweep through HBM); with the default grid and tiles
+   below, and instances of 16 nodes a side or more, an even number of the launches
+   of a call advance four steps each instead, the states being equal bit for bit.
+   Set before capturing a graph. */
 int lbm_ensemble_configure(lbm_ensemble e, int steps_per_pass);
 /* Grid of the two-step launches: persistent = 0 (default) launches one block
    per tile of the union tile list (all instances in one launch, the hardware

@@ -18,7 +18,8 @@ size_t up256(size_t x) { return (x + 255) & ~size_t(255); }
 struct EnsLayout {
     size_t off_inst = 0, off_tiles = 0, off_tiles2 = 0, off_tiles2p = 0, off_err = 0, off_partials = 0, off_tbegin = 0,
            total = 0;
-    int ntiles = 0, ntiles2 = 0, ntiles2p = 0;
+    size_t off_items4 = 0;
+    int ntiles = 0, ntiles2 = 0, ntiles2p = 0, nitems4 = 0, rows4 = 0;
     std::vector<size_t> off_pop;    // per instance: buffer A offset (B follows)
     std::vector<long long> pitch;
 };
@@ -38,6 +39,18 @@ int ens_layout(int count, const int *nx, const int *ny, EnsLayout *L)
     L->ntiles = (int)tiles;
     L->ntiles2 = (int)tiles2;
     L->ntiles2p = (int)tiles2p;
+    // strips of the four-step sweeps, cut into chunks of about rows4 rows: some three
+    // waves of four blocks on 152 SMs, 32 to 128 rows (a chunk takes 9 iterations more)
+    long long strip_rows = 0, items4 = 0;
+    bool fits4 = true;
+    for (int i = 0; i < count; ++i) {
+        strip_rows += (long long)((nx[i] + kEns4Cols - 1) / kEns4Cols) * ny[i];
+        if (nx[i] < 16 || ny[i] < 16) fits4 = false;
+    }
+    L->rows4 = (int)std::min(128LL, std::max(32LL, strip_rows / 1824));
+    for (int i = 0; i < count && fits4; ++i)
+        items4 += (long long)((nx[i] + kEns4Cols - 1) / kEns4Cols) * ((ny[i] + L->rows4 - 1) / L->rows4);
+    L->nitems4 = (int)items4;
     size_t off = 0;
     L->off_inst = off;
     off += up256(sizeof(EnsInst) * (size_t)count);
@@ -47,6 +60,8 @@ int ens_layout(int count, const int *nx, const int *ny, EnsLayout *L)
     off += up256(sizeof(int4) * (size_t)tiles2);
     L->off_tiles2p = off;
     off += up256(sizeof(int4) * (size_t)tiles2p);
+    L->off_items4 = off;
+    off += up256(sizeof(int4) * (size_t)items4);
     L->off_err = off;                   // error word at +0, tile-claim counters at +128
     off += 256;
     L->off_partials = off;
@@ -169,6 +184,17 @@ int lbm_ensemble_create(lbm_ensemble *out, int count, const int *nx, const int *
         for (int ty = 0; ty < ny[i]; ty += kEns2PRows)
             for (int tx = 0; tx < nx[i]; tx += kEns2PCols) tiles2p.push_back(make_int4(i, tx, ty, 0));
     }
+    std::vector<int4> items4;
+    if (L.nitems4 > 0)
+        for (int i : by_size) {
+            const int chunks = (ny[i] + L.rows4 - 1) / L.rows4, H = (ny[i] + chunks - 1) / chunks;
+            for (int y = 0; y < ny[i]; y += H)
+                for (int x = 0; x < nx[i]; x += kEns4Cols) items4.push_back(make_int4(i, x, y, std::min(y + H, ny[i])));
+        }
+    // tallest strips first, whatever instance they belong to
+    std::stable_sort(items4.begin(), items4.end(), [](const int4 &a, const int4 &b) { return a.w - a.z > b.w - b.z; });
+    e->nitems4 = (int)items4.size();
+    e->d_items4 = (int4 *)(ws + L.off_items4);
     e->ntiles2 = (int)tiles2.size();
     e->d_tiles2 = (int4 *)(ws + L.off_tiles2);
     e->ntiles2p = (int)tiles2p.size();
@@ -188,6 +214,10 @@ int lbm_ensemble_create(lbm_ensemble *out, int count, const int *nx, const int *
                                              cudaMemcpyHostToDevice, st), "lbm_ensemble_create two-step tile table");
     if (!rc) rc = cuda_check(cudaMemcpyAsync(e->d_tiles2p, tiles2p.data(), sizeof(int4) * tiles2p.size(),
                                              cudaMemcpyHostToDevice, st), "lbm_ensemble_create pair tile table");
+    if (!rc && e->nitems4 > 0)
+        rc = cuda_check(cudaMemcpyAsync(e->d_items4, items4.data(), sizeof(int4) * items4.size(), cudaMemcpyHostToDevice, st),
+                        "lbm_ensemble_create strip table");
+    if (!rc && e->nitems4 > 0) rc = cuda_check(ens_launch_step4(e, true, st), "lbm_ensemble_create kernel attributes");
     if (!rc) rc = cuda_check(cudaMemsetAsync(e->err, 0, 256, st), "lbm_ensemble_create error word and counters");
     if (!rc) rc = cuda_check(cudaMemcpyAsync(e->d_tiles, tiles.data(), sizeof(int4) * tiles.size(),
                                              cudaMemcpyHostToDevice, st), "lbm_ensemble_create tile table");
@@ -241,6 +271,14 @@ int lbm_ensemble_set_phi(lbm_ensemble e, const void *dev_phi, int prec, void *st
     return cuda_check(ens_launch_init(e, dev_phi, prec, (cudaStream_t)stream), "lbm_ensemble_set_phi");
 }
 
+// how many sweeps of four steps serve a call: with two steps per pass and the
+// default launch (one block per piece of work, 30 x 30 tiles), an even number
+static int fours(const lbm_ensemble_s *e, int mode, int nsteps)
+{
+    if (mode != 0 || e->spp != 2 || e->persistent2 != 0 || e->shape2 != 0 || e->nitems4 == 0) return 0;
+    return nsteps / 8 * 2;
+}
+
 int lbm_ensemble_step(lbm_ensemble e, int nsteps, int mode, void *stream)
 {
     if (!e) return fail(LBM_EINVAL, "null ensemble");
@@ -248,6 +286,11 @@ int lbm_ensemble_step(lbm_ensemble e, int nsteps, int mode, void *stream)
     if (mode != 0 && mode != 1) return fail(LBM_EINVAL, "mode must be 0 (persistent) or 1 (one launch per instance)");
     cudaStream_t st = (cudaStream_t)stream;
     int n = 0;
+    // sweeps of four in pairs: the launches of a call stay even or odd in number
+    for (int four = fours(e, mode, nsteps); four > 0; --four, n += 4) {
+        if (int rc = cuda_check(ens_launch_step4(e, false, st), "lbm_ensemble_step (four steps per sweep)")) return rc;
+        e->parity ^= 1;
+    }
     if (mode == 0 && e->spp == 2)
         for (; n + 2 <= nsteps; n += 2) {
             if (int rc = cuda_check(ens_launch_step2(e, st), "lbm_ensemble_step (two steps per pass)")) return rc;
@@ -307,7 +350,12 @@ int lbm_ensemble_capture(lbm_ensemble e, int nsteps, void *stream)
     if (int rc = cuda_check(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal), "cudaStreamBeginCapture"))
         return rc;
     int rc = LBM_OK;
-    for (int n = 0; n < nsteps && !rc; n += e->spp) {
+    int n = 0;
+    for (int four = fours(e, 0, nsteps); four > 0 && !rc; --four, n += 4) {
+        rc = cuda_check(ens_launch_step4(e, false, st), "captured step");
+        e->parity ^= 1;
+    }
+    for (; n < nsteps && !rc; n += e->spp) {
         rc = cuda_check(e->spp == 2 ? ens_launch_step2(e, st) : ens_launch_step(e, 0, e->ntiles, e->grid, st),
                         "captured step");
         e->parity ^= 1;

@@ -154,7 +154,8 @@ template <int K = 0, class F> __device__ __forceinline__ void each_k(F f)
 // One strip. EDGE: it touches the edges of the grid -- `cols`, its columns wrap or meet
 // walls; `rows`, it has rows at anti-bounce-back walls.
 template <int CONV, int DIFF, int SRC, bool KF, int T, int KW, int P, int ST, bool EDGE>
-__device__ __forceinline__ void march_strip(const MarchArgs &a, float *sm, int X0, int Y0, int Y1, bool cols, bool rows)
+__device__ __forceinline__ void march_strip(const MarchArgs &a, const Coll<F2> &kc, float *sm, int X0, int Y0, int Y1,
+                                            bool cols, bool rows)
 {
     using M = March<T, KW, P, ST>;
     if (!EDGE) cols = rows = false;
@@ -218,7 +219,7 @@ __device__ __forceinline__ void march_strip(const MarchArgs &a, float *sm, int X
             A35 = F2(__ldg(a.Afield + a.plane + i0), __ldg(a.Afield + a.plane + i1));
             A5 = F2(__ldg(a.Afield + 2 * a.plane + i0), __ldg(a.Afield + 2 * a.plane + i1));
         }
-        relax<F2, CONV, DIFF, KF, SRC>(a.k, a.has_src != 0, g, A3, A35, A5, ph);
+        relax<F2, CONV, DIFF, KF, SRC>(kc, a.has_src != 0, g, A3, A35, A5, ph);
     };
 
     // Level 0's input. The nine planes' rows that row r pulls from (columns X0 - T and on) are
@@ -418,8 +419,8 @@ k_march(const __grid_constant__ MarchArgs a)
     // without cols no pull leaves the row, and the bulk copies end in the row or its padding
     const bool cols = X0 - T < 0 || X0 - (T - 1) + M::kW >= a.nx || X0 - T + M::kInW > a.pitch;
     const bool rows = a.abb_y && (Y0 - T < 0 || Y1 + T > a.ny);
-    if (cols || rows) march_strip<CONV, DIFF, SRC, KF, T, KW, P, ST, true>(a, sm_m, X0, Y0, Y1, cols, rows);
-    else march_strip<CONV, DIFF, SRC, KF, T, KW, P, ST, false>(a, sm_m, X0, Y0, Y1, false, false);
+    if (cols || rows) march_strip<CONV, DIFF, SRC, KF, T, KW, P, ST, true>(a, a.k, sm_m, X0, Y0, Y1, cols, rows);
+    else march_strip<CONV, DIFF, SRC, KF, T, KW, P, ST, false>(a, a.k, sm_m, X0, Y0, Y1, false, false);
 }
 
 // Blocks: one wave of four per SM, or up to three where the chunks stay 48 rows or

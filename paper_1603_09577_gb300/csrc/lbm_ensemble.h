@@ -45,6 +45,8 @@ struct lbm_ensemble_s {
     int shape2 = 0;                 // two-step tiles: 0 30 x 30 (one node per thread), 1 62 x 14 (two)
     int persistent2 = 0;            // two-step launch: 0 a block per tile, 1 persistent with a fixed
                                     // stride, 2 persistent with tiles claimed from a counter
+    int nitems4 = 0;                // strips of the four-step sweeps; 0: an instance is too small for them
+    int4 *d_items4 = nullptr;       // instance, first column, rows from .. to
     int4 *d_tiles2 = nullptr;
     int4 *d_tiles2p = nullptr;
     int *d_claim = nullptr;         // tile counter and departed-block counter of mode 2
@@ -63,6 +65,9 @@ struct lbm_ensemble_s {
 namespace lbm {
 cudaError_t ens_launch_step(const lbm_ensemble_s *e, int t_begin, int t_end, int blocks, cudaStream_t st);
 cudaError_t ens_launch_step2(const lbm_ensemble_s *e, cudaStream_t st);
+// four steps over the strips of every instance (kernels_ensemble4.cu)
+cudaError_t ens_launch_step4(const lbm_ensemble_s *e, bool prepare, cudaStream_t st);
+constexpr int kEns4Cols = 120;      // output columns of a strip
 int ens2_occupancy_blocks(int family, int shape);
 constexpr int kEns2Tile = 30;       // two-step tiles: 30 x 30 outputs
 constexpr int kEns2PCols = 62;      // two-step pair tiles: 62 x 14 outputs
