@@ -54,12 +54,6 @@ template <class R> __host__ __device__ __forceinline__ int tile_rx(int W, int T)
     return (W + 2 * (T - 1) + N - 1) / N * N;
 }
 
-// whether the region of T steps fits a plane
-template <class R> inline bool tile_fits(int W, int H, int T)
-{
-    return (long long)tile_rx<R>(W, T) * (H + 2 * (T - 1)) + kTilePad <= kTilePlane<R>;
-}
-
 __device__ __forceinline__ int tile_wrap(int v, int n)
 {
     v %= n;

@@ -275,6 +275,39 @@ static int device_sms(lbm_solver *s)
     return cuda_check(cudaDeviceGetAttribute(&s->sms, cudaDevAttrMultiProcessorCount, dev), "SM count");
 }
 
+// As few launches of the plan's tiles as hold nsteps, even or odd in number as with
+// steps_per_pass steps each (a captured call then ends on the buffer it started from)
+static int tile_launches(const lbm_solver *s, int nsteps)
+{
+    const int wanted = s->d.steps_per_pass == 2 ? nsteps / 2 + nsteps % 2 : nsteps;
+    const int launches = (nsteps + s->plan.T - 1) / s->plan.T;
+    return ((launches ^ wanted) & 1) && launches < nsteps ? launches + 1 : launches;
+}
+
+// The general path's small lattices (the C-free variant runs one step per launch).
+// Measured on the Burgers-Fisher problem, us per step, other kernel -> tiles: FP32 one
+// step per pass 60^2 4.4 -> 2.0, 301^2 6.4 -> 4.1, 500^2 8.5 -> 7.0, 700^2 10.6 -> 12.7; two
+// 6.4 -> 1.9, 6.4 -> 4.1, 7.7 -> 7.0, 9.8 -> 12.7; FP64 60^2 24.9 -> 11.1, 200^2 45.4 -> 28.1,
+// 500^2 103 -> 97, 700^2 174 -> 165 (there with one step per launch: smaller blocks).
+static bool tile_general_wanted(lbm_solver *s)
+{
+    if (s->d.kernel_variant != 0 || s->d.block_rows != 0 || s->c.cfree || s->d.prec == LBM_BF16S || s->c.conv > 2) return false;
+    if ((long long)s->d.nx * s->d.ny > (s->d.prec == LBM_F64 ? 500000 : 250000)) return false;
+    if (s->plan.T == 0) s->plan = tile_plan(s->d.nx, s->d.ny, s->d.prec == LBM_F64, true, s->sms);
+    return s->d.prec == LBM_F64 || s->plan.T >= 2;
+}
+
+static cudaError_t launch_tile_general(const lbm_solver *s, int src, const double *records, int steps, bool prepare,
+                                       cudaStream_t st)
+{
+    const bool a = s->d.scheme == LBM_SCHEME_A;
+    if (s->d.prec == LBM_F64)
+        return a ? launch_tile_general_f64_a(s, src, records, steps, prepare, st)
+                 : launch_tile_general_f64_b(s, src, records, steps, prepare, st);
+    return a ? launch_tile_general_f32_a(s, src, records, steps, prepare, st)
+             : launch_tile_general_f32_b(s, src, records, steps, prepare, st);
+}
+
 // nsteps as sweeps of four, two and one steps. The number of launches stays odd or
 // even as it is with steps_per_pass steps each (n, or n/2 + n%2), so that a
 // captured call that ended on the buffer it started from still does: with m pairs
@@ -282,13 +315,10 @@ static int device_sms(lbm_solver *s)
 static int step_auto(lbm_handle h, int nsteps, cudaStream_t st)
 {
     if (int rc = device_sms(h)) return rc;
-    if (h->plan.T == 0) h->plan = tile_plan(h->d.nx, h->d.ny, h->d.prec == LBM_F64, h->sms);
+    if (h->plan.T == 0) h->plan = tile_plan(h->d.nx, h->d.ny, h->d.prec == LBM_F64, false, h->sms);
     if (tile_wanted(h)) {
         if (int rc = cuda_check(launch_tile(h, h->cur, 1, true, st), "lbm_step (kernel attributes)")) return rc;
-        // as few launches as hold nsteps, even or odd in number as promised, of nearly equal size
-        const int wanted = h->d.steps_per_pass == 2 ? nsteps / 2 + nsteps % 2 : nsteps;
-        int launches = (nsteps + h->plan.T - 1) / h->plan.T;
-        if (((launches ^ wanted) & 1) && launches < nsteps) ++launches;
+        const int launches = tile_launches(h, nsteps);
         for (int i = 0, done = 0; i < launches; ++i) {
             const int steps = (nsteps - done) / (launches - i) + ((nsteps - done) % (launches - i) != 0);
             if (int rc = cuda_check(launch_tile(h, h->cur, steps, false, st), "lbm_step (small lattice)")) return rc;
@@ -449,6 +479,7 @@ int lbm_set_coeffs(lbm_handle h, const lbm_coeffs *c)
         if (!relax_block(c->K, &a, &b, &d)) return fail(LBM_EINVAL, "K is not symmetric positive definite");
     }
     h->c = *c;
+    h->plan.T = 0;                       // the family decides which kernels serve it
     h->coeffs_set = 1;
     return LBM_OK;
 }
@@ -534,6 +565,22 @@ int lbm_step(lbm_handle h, int nsteps, void *stream)
         const double *records = nee ? h->dir_vals : nullptr;
         if (nee)
             if (int rc = flush_record_reset(h, st)) return rc;
+        if (int rc = device_sms(h)) return rc;
+        if (tile_general_wanted(h)) {
+            if (int rc = cuda_check(launch_tile_general(h, h->cur, records, 1, true, st), "lbm_step (kernel attributes)"))
+                return rc;
+            const int launches = tile_launches(h, nsteps);
+            for (int i = 0; i < launches; ++i) {
+                const int left = launches - i, steps = (nsteps - done + left - 1) / left;
+                h->dir_off = done;
+                if (int rc = cuda_check(launch_tile_general(h, h->cur, records, steps, false, st),
+                                        "lbm_step (general, small lattice)"))
+                    return rc;
+                h->cur ^= 1;
+                h->t += steps;
+                done += steps;
+            }
+        }
         if (h->d.steps_per_pass == 2) {
             for (; done + 2 <= nsteps; done += 2) {
                 h->dir_off = done;

@@ -176,7 +176,14 @@ cudaError_t launch_march_src(const lbm_solver *s, int src, bool prepare, cudaStr
 cudaError_t launch_march_free(const lbm_solver *s, int src, bool prepare, cudaStream_t st);
 cudaError_t launch_march_kfield(const lbm_solver *s, int src, bool prepare, cudaStream_t st);
 // `steps` steps in one launch over the tiles of s->plan (kernels_tile.cuh)
-TilePlan tile_plan(int nx, int ny, bool f64, int sms);
+TilePlan tile_plan(int nx, int ny, bool f64, bool general, int sms);
+#define LBM_DECLARE_TILE_GENERAL(NAME) \
+    cudaError_t NAME(const lbm_solver *s, int src, const double *records, int steps, bool prepare, cudaStream_t st)
+LBM_DECLARE_TILE_GENERAL(launch_tile_general_f32_a);
+LBM_DECLARE_TILE_GENERAL(launch_tile_general_f32_b);
+LBM_DECLARE_TILE_GENERAL(launch_tile_general_f64_a);
+LBM_DECLARE_TILE_GENERAL(launch_tile_general_f64_b);
+#undef LBM_DECLARE_TILE_GENERAL
 cudaError_t launch_tile_f32_const(const lbm_solver *s, int src, int steps, bool prepare, cudaStream_t st);
 cudaError_t launch_tile_f32_kfield(const lbm_solver *s, int src, int steps, bool prepare, cudaStream_t st);
 cudaError_t launch_tile_f64_const(const lbm_solver *s, int src, int steps, bool prepare, cudaStream_t st);

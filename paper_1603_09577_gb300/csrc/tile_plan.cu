@@ -1,5 +1,5 @@
 // tile_plan.cu -- tiles and steps per launch of the small lattices' kernel.
-#include "kernels_tile.cuh"
+#include "kernels_tile_general.cuh"
 
 namespace lbm {
 
@@ -10,26 +10,29 @@ namespace lbm {
 // four warps (68 to 78 operations of 64 cycles, one warp per quarter of the SM).
 // Fitted to measured launches (us): FP32 100^2 T = 8 8.5, 400^2 T = 4 10.4, T = 8 17.4, 600^2
 // T = 4 16.7, T = 8 32; FP64 64^2 T = 3 10.5, 128^2 T = 2 10.4, T = 4 24.9, 200^2 T = 2 18.6.
-TilePlan tile_plan(int nx, int ny, bool f64, int sms)
+TilePlan tile_plan(int nx, int ny, bool f64, bool general, int sms)
 {
     TilePlan best;
     best.us = 1e30;
     for (int T = 1; T <= kTileMaxT; ++T)
         for (int bx = 1; bx <= nx && bx <= 4 * sms; ++bx) {
             const int W = (nx + bx - 1) / bx;
-            if ((nx + W - 1) / W != bx) continue;
+            if ((nx + W - 1) / W != bx || (general && W < 2)) continue;
             for (int waves = 1; waves <= 4; ++waves) {
                 const int by = std::min(ny, waves * sms / bx);
                 if (by < 1) continue;
-                const int H = (ny + by - 1) / by, N = f64 ? 1 : 2;
-                const int RX = f64 ? tile_rx<double>(W, T) : tile_rx<float>(W, T), RY = H + 2 * (T - 1);
-                if (T > 1 ? !(f64 ? tile_fits<double>(W, H, T) : tile_fits<float>(W, H, T)) : (long long)RX * RY >= 65536)
-                    continue;
+                const int H = (ny + by - 1) / by, N = f64 || general ? 1 : 2;
+                const int RX = f64 || general ? tile_rx<double>(W, T) : tile_rx<float>(W, T), RY = H + 2 * (T - 1);
+                if (general && H < 2) continue;
+                const int plane = general ? (f64 ? kTileGPlane<double> : kTileGPlane<float>)
+                                          : (f64 ? kTilePlane<double> : kTilePlane<float>);
+                if ((long long)RX * RY + kTilePad > (T > 1 ? plane : 65536)) continue;
                 const int n_waves = (bx * ((ny + H - 1) / H) + sms - 1) / sms;
                 double t = 0.0;
                 for (int l = 1; l <= T; ++l) {                   // rows drop out whole, columns do not
                     const int warps = (RX / N * (RY - 2 * (l - 1)) + 31) / 32;
-                    t += f64 ? 0.2 + 2.2 * ((warps + 3) / 4) : 0.25 + 0.055 * warps;
+                    if (general) t += f64 ? 0.3 + 4.6 * ((warps + 3) / 4) : 0.4 + 0.06 * warps;
+                    else t += f64 ? 0.2 + 2.2 * ((warps + 3) / 4) : 0.25 + 0.055 * warps;
                 }
                 const double us = ((f64 ? 3.0 : 4.5) + n_waves * t) / T;
                 if (us < best.us) best = TilePlan{W, H, T, us};
