@@ -391,7 +391,7 @@ __device__ __forceinline__ void pull3_node(const Params3<typename St3<PREC>::C> 
                 if (p.abb[0] && (xs < 0 || xs >= p.nx)) { tot += xs < 0 ? p.phi_wall[0] : p.phi_wall[1]; ++cnt; }
                 if (p.abb[1] && (ys < 0 || ys >= p.ny)) { tot += ys < 0 ? p.phi_wall[2] : p.phi_wall[3]; ++cnt; }
                 if (p.abb[2] && (zs < 0 || zs >= p.nz)) { tot += zs < 0 ? p.phi_wall[4] : p.phi_wall[5]; ++cnt; }
-                if (PREC == LBM_F32) {
+                if (PREC != LBM_BF16S) {
                     const int set = (p.abb[0] && (xs < 0 || xs >= p.nx) ? 1 : 0) |
                                     (p.abb[1] && (ys < 0 || ys >= p.ny) ? 2 : 0) |
                                     (p.abb[2] && (zs < 0 || zs >= p.nz) ? 4 : 0);

@@ -1,4 +1,4 @@
-// lbm3_relax.cuh -- the D3Q19 collision of the FP32 kernels, every operation with its
+// lbm3_relax.cuh -- the D3Q19 collision of the FP32 and FP64 kernels, every operation with its
 // rounding written out (as relax() of lbm_relax.cuh, and by its two rules: a product
 // that meets a sum is a fused multiply-add), so that the one-step kernel and the
 // two-step sweeps return the same bits. It is the projector form of collide3() with
