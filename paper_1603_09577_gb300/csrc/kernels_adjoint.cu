@@ -247,14 +247,26 @@ k_adjoint_end(const Params<C> p, const void *__restrict__ phi0, int in_prec, con
     block_add2(dux, duy, partials + 2 * ((size_t)blockIdx.y * gridDim.x + blockIdx.x));
 }
 
-// sum of the per-block u-gradient partials in block order
-__global__ void k_adjoint_du(const double *__restrict__ partials, int nb, double *__restrict__ du)
+// sum of the per-block u-gradient partials: each thread a strided share, then a
+// fixed-order tree (one thread over all of them took 1024 dependent additions at 512^2)
+constexpr int kDuThreads = 256;
+__global__ void __launch_bounds__(kDuThreads) k_adjoint_du(const double *__restrict__ partials, int nb, double *__restrict__ du)
 {
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
-        double a = 0.0, b = 0.0;
-        for (int q = 0; q < nb; ++q) { a += partials[2 * q]; b += partials[2 * q + 1]; }
-        du[0] = a;
-        du[1] = b;
+    __shared__ double sa[kDuThreads], sb[kDuThreads];
+    double a = 0.0, b = 0.0;
+    for (int q = threadIdx.x; q < nb; q += kDuThreads) { a += partials[2 * q]; b += partials[2 * q + 1]; }
+    sa[threadIdx.x] = a;
+    sb[threadIdx.x] = b;
+    for (int off = kDuThreads / 2; off > 0; off >>= 1) {
+        __syncthreads();
+        if ((int)threadIdx.x < off) {
+            sa[threadIdx.x] += sa[threadIdx.x + off];
+            sb[threadIdx.x] += sb[threadIdx.x + off];
+        }
+    }
+    if (threadIdx.x == 0) {
+        du[0] = sa[0];
+        du[1] = sb[0];
     }
 }
 
@@ -301,7 +313,7 @@ cudaError_t launch_adjoint_end(const lbm_solver *s, const void *phi0, int in_pre
                                                      dphi0, dK, partials);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    k_adjoint_du<<<1, 32, 0, st>>>(partials, adjoint_blocks(s), du);
+    k_adjoint_du<<<1, kDuThreads, 0, st>>>(partials, adjoint_blocks(s), du);
     return cudaGetLastError();
 }
 
