@@ -10,13 +10,21 @@
 
 namespace lbm {
 
-template <int PREC, int CONV, int DIFF>
+// KF: a per-node tensor field, a kernel of its own, since in FP32 it takes another
+// collision and other walls. 2636 x 1533, conv 0, FP32: 5,003 us per pass; with both
+// collisions in one kernel and the walls of both from the table 5,432, with collide()
+// and wall_term() for both 5,067.
+template <int PREC, int CONV, int DIFF, bool KF>
 __global__ void __launch_bounds__(256)
 k_step(const Params<typename Store<PREC>::C> p, const typename Store<PREC>::T *__restrict__ src,
        const float *__restrict__ src_phi, typename Store<PREC>::T *__restrict__ dst, float *__restrict__ dst_phi)
 {
     using S = Store<PREC>;
     using C = typename S::C;
+    // FP32 with a per-node tensor keeps collide() and wall_term(): these are the forward
+    // states of the adjoint, whose gradient in u is a sum of cancelling terms that
+    // magnifies a change of the last bit
+    constexpr int NP = KF && PREC == LBM_F32 ? LBM_BF16S : PREC;
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
     if (x >= p.nx || y >= p.ny) return;
@@ -55,17 +63,14 @@ k_step(const Params<typename Store<PREC>::C> p, const typename Store<PREC>::T *_
             const bool ox = p.abb_x && (xs < 0 || xs >= p.nx);
             const bool oy = p.abb_y && (ys < 0 || ys >= p.ny);
             if (ox || oy) {
-                f[k] = wall_value<PREC, C, CONV, DIFF>(p, k, ox, oy) - S::ld(src + opp(k) * P, own, src_phi, wgt<C>(opp(k)));
+                f[k] = wall_value<NP, C, CONV, DIFF>(p, k, ox, oy) - S::ld(src + opp(k) * P, own, src_phi, wgt<C>(opp(k)));
             }
         }
     }
 
     C phi;
-    // (FP32 with a per-node tensor keeps collide(): these are the forward states of the
-    // adjoint, whose gradient in u is a sum of cancelling terms that magnifies a change
-    // of the last bit)
-    if (p.Afield)
-        collide_stored<PREC == LBM_F32 ? LBM_BF16S : PREC, C, CONV, DIFF, true>(
+    if constexpr (KF)
+        collide_stored<NP, C, CONV, DIFF, true>(
             p, f, __ldg(p.Afield + own), __ldg(p.Afield + P + own), __ldg(p.Afield + 2 * P + own), phi);
     else
         collide_stored<PREC, C, CONV, DIFF, false>(p, f, p.A3, p.A35, p.A5, phi);
@@ -83,7 +88,8 @@ static cudaError_t step_t(const lbm_solver *s, const void *src, const float *src
     const int by = s->d.block_rows > 0 ? s->d.block_rows : 8;
     dim3 block(32, by);
     dim3 grid((s->d.nx + 31) / 32, (s->d.ny + by - 1) / by);
-    k_step<PREC, CONV, DIFF><<<grid, block, 0, st>>>(p, (const T *)src, src_h, (T *)dst, dst_h);
+    if (p.Afield) k_step<PREC, CONV, DIFF, true><<<grid, block, 0, st>>>(p, (const T *)src, src_h, (T *)dst, dst_h);
+    else k_step<PREC, CONV, DIFF, false><<<grid, block, 0, st>>>(p, (const T *)src, src_h, (T *)dst, dst_h);
     return cudaGetLastError();
 }
 
