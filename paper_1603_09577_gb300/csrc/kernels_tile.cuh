@@ -51,7 +51,8 @@ template <class R> constexpr int kTilePlane = kTileSmem / (18 * (int)sizeof(R));
 template <class R> __host__ __device__ __forceinline__ int tile_rx(int W, int T)
 {
     constexpr int N = TileVec<R>::N;
-    return (W + 2 * (T - 1) + N - 1) / N * N;
+    const int rx = (W + 2 * (T - 1) + N - 1) / N * N;
+    return rx < 2 * N ? 2 * N : rx;                  // two items a row at least: the division by a multiply
 }
 
 __device__ __forceinline__ int tile_wrap(int v, int n)

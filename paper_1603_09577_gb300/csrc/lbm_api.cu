@@ -294,7 +294,7 @@ static bool tile_general_wanted(lbm_solver *s)
     if (s->d.kernel_variant != 0 || s->d.block_rows != 0 || s->c.cfree || s->d.prec == LBM_BF16S || s->c.conv > 2) return false;
     if ((long long)s->d.nx * s->d.ny > (s->d.prec == LBM_F64 ? 500000 : 250000)) return false;
     if (s->plan.T == 0) s->plan = tile_plan(s->d.nx, s->d.ny, s->d.prec == LBM_F64, true, s->sms);
-    return s->d.prec == LBM_F64 || s->plan.T >= 2;
+    return s->plan.us < 1e29 && (s->d.prec == LBM_F64 || s->plan.T >= 2);
 }
 
 static cudaError_t launch_tile_general(const lbm_solver *s, int src, const double *records, int steps, bool prepare,

@@ -34,8 +34,8 @@ namespace lbm {
 // Launch of a small lattice: W x H tiles, T steps per launch (kernels_tile.cuh); us:
 // the estimated time of a step. T = 0: not planned yet.
 struct TilePlan {
-    int W, H, T;
-    double us;
+    int W = 0, H = 0, T = 0;
+    double us = 0.0;
 };
 
 }  // namespace lbm

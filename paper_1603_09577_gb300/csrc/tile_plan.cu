@@ -12,18 +12,16 @@ namespace lbm {
 // T = 4 16.7, T = 8 32; FP64 64^2 T = 3 10.5, 128^2 T = 2 10.4, T = 4 24.9, 200^2 T = 2 18.6.
 TilePlan tile_plan(int nx, int ny, bool f64, bool general, int sms)
 {
-    TilePlan best;
-    best.us = 1e30;
+    TilePlan best{nx, ny, 1, 1e30};                  // no tiling fits: never the fastest
     for (int T = 1; T <= kTileMaxT; ++T)
         for (int bx = 1; bx <= nx && bx <= 4 * sms; ++bx) {
             const int W = (nx + bx - 1) / bx;
             if ((nx + W - 1) / W != bx || (general && W < 2)) continue;
             for (int waves = 1; waves <= 4; ++waves) {
-                const int by = std::min(ny, waves * sms / bx);
+                const int by = std::min(general ? ny / 2 : ny, waves * sms / bx);
                 if (by < 1) continue;
                 const int H = (ny + by - 1) / by, N = f64 || general ? 1 : 2;
                 const int RX = f64 || general ? tile_rx<double>(W, T) : tile_rx<float>(W, T), RY = H + 2 * (T - 1);
-                if (general && H < 2) continue;
                 const int plane = general ? (f64 ? kTileGPlane<double> : kTileGPlane<float>)
                                           : (f64 ? kTilePlane<double> : kTilePlane<float>);
                 if ((long long)RX * RY + kTilePad > (T > 1 ? plane : 65536)) continue;

@@ -19,7 +19,9 @@ CASES = [(2, 2, (0, 0), 0, (0.05, -0.03), 0, 0.0), (3, 5, (1, 1), 1, (0.08, 0.05
          (64, 64, (0, 0), 0, (0.05, 0.02), 1, -0.01), (131, 65, (1, 1), 1, (0.04, 0.05), 0, -0.01),
          (128, 128, (0, 0), 0, (0.05, 0.04), 0, 0.0), (199, 201, (0, 1), 0, (0.0, 0.0), 0, 0.0),
          (401, 300, (1, 0), 0, (0.0, 0.0), 1, 0.0), (2000, 7, (1, 1), 1, (0.05, 0.05), 2, 0.0),
-         (400, 400, (0, 0), 1, (0.05, 0.05), 1, 0.0), (33, 1500, (0, 0), 0, (0.02, 0.05), 2, -0.01)]
+         (400, 400, (0, 0), 1, (0.05, 0.05), 1, 0.0), (33, 1500, (0, 0), 0, (0.02, 0.05), 2, -0.01),
+         (2, 900, (0, 1), 0, (0.02, 0.05), 1, 0.0), (900, 2, (1, 0), 1, (0.02, 0.05), 1, 0.0),
+         (4, 1500, (0, 0), 1, (0.05, 0.05), 0, 0.0)]
 IDS = [f"{c[0]}x{c[1]}-bc{c[2][0]}{c[2][1]}-c{c[3]}d{c[5]}" for c in CASES]
 
 

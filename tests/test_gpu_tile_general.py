@@ -16,7 +16,8 @@ BCN = {0: "periodic", 1: "abb", 2: "nee"}
 # carry it at most linearly, a few hundred units of rounding at the field's scale
 TOL = {"f64": 30 * 16 * 2.0 ** -53, "f32": 30 * 16 * 2.0 ** -24}
 CASES = [(3, 3, (2, 2)), (3, 40, (2, 0)), (61, 5, (0, 2)), (64, 64, (2, 2)), (133, 71, (2, 2)), (97, 130, (1, 1)),
-         (301, 301, (2, 2)), (160, 33, (2, 0)), (50, 50, (0, 0))]
+         (301, 301, (2, 2)), (160, 33, (2, 0)), (50, 50, (0, 0)),
+         (3, 5, (2, 2)), (2, 2, (0, 0)), (2, 3, (1, 0)), (2, 900, (0, 1)), (900, 3, (0, 2))]
 COEF = dict(conv=2, power=2, u=(0.06, -0.03), diff=1, K=(0.02, 0.008, 0.01))
 
 
