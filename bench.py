@@ -185,6 +185,19 @@ def clocks_summary(proc):
     return {"sm_mhz": statistics.median(mhz), "sm_max_mhz": maxm, "reasons": sorted(reasons), "samples": len(mhz)}
 
 
+def ensemble_launches(nsteps, spp, cfg, inst):
+    """Step launches of a captured 100-step ensemble graph replayed over nsteps steps,
+    and their kernel: with two steps per pass and the default launch large ensembles
+    advance four steps per sweep, in pairs of sweeps."""
+    cols = sum(-(-d["nx"] // 120) * 120 * d["ny"] for d in inst)
+    if (spp == 2 and not cfg.get("persistent") and not cfg.get("pair_tiles") and cols >= 4000000
+            and all(d["nx"] >= 16 and d["ny"] >= 16 for d in inst)):
+        return nsteps // 100 * (24 + 2), "k_ens_march (four steps per sweep, graph-replayed)", 4
+    if spp == 2:
+        return nsteps // 2, f"k_ens_step2 (two steps per launch, graph-replayed, autotuned launch {cfg})", 2
+    return nsteps, "k_ens_step (persistent, graph-replayed)", 1
+
+
 def measured_peak():
     try:
         with open(os.path.join(ROOT, "MEASURED_PEAKS.json")) as f:
@@ -206,10 +219,36 @@ def traffic_per_launch(kernel_sha, key="k_step2"):
         return None
 
 
-def step_kernel(prec, spp, variant):
+def takes_march(prec, variant, rows, nx, ny):
+    """Whether this launch configuration's sweeps advance four time steps (the
+    library's choice for FP32 where it is left the launch and the lattice is large)."""
+    return (prec == "f32" and (variant, rows) in ((0, 0), (5, 4)) and nx >= 128 and ny >= 64
+            and nx * ny >= 1 << 18)
+
+
+def step_launches(nsteps, prec, spp, variant, rows, nx, ny):
+    """Step-kernel launches of one lbm_step(nsteps) call (on lattices of fewer than
+    2^18 nodes, where one launch may take up to eight steps, at most these)."""
+    if not takes_march(prec, variant, rows, nx, ny):
+        return nsteps // spp + nsteps % spp
+    # sweeps of four, then of two, then single steps; with two steps per pass an even
+    # number of fours, with one as many launches, modulo 2, as steps
+    twos, one = nsteps // 2, nsteps % 2
+    four = twos // 2
+    if four & 1 != (0 if spp == 2 else twos & 1):
+        four = max(0, four - 1)
+    two = twos - 2 * four
+    if spp == 1 and (four + two) & 1:
+        two, one = two - 1, one + 2
+    return four + two + one
+
+
+def step_kernel(prec, spp, variant, rows, nx, ny):
     """Name of the step kernel a launch configuration runs, and its DRAM bytes per
     launch from the committed ncu capture (None when there is none or the
     kernel's sources changed since)."""
+    if takes_march(prec, variant, rows, nx, ny):
+        return "k_march (four fused pull-stream + collide steps per sweep)", None
     if spp == 2 and variant == 5:
         return ("k_step2p (two fused pull-stream + collide steps per sweep, pair tiles)",
                 traffic_per_launch(src_sha(PAIR_SRC), f"k_step2p_{prec}"))
@@ -371,7 +410,8 @@ def run_ensemble(args):
     else:
         nodes_r0 = nodes
     peak, src = measured_peak()
-    achieved = 72.0 * nodes_r0 * (steps // args.ens_spp) / (ms_graph / 1e3) / 1e9
+    ens_launches, ens_kernel, ens_steps = ensemble_launches(steps, args.ens_spp, cfg, inst)
+    achieved = 72.0 * nodes_r0 * ens_launches / (ms_graph / 1e3) / 1e9
     out = {"metric": "MLUPS", "value": val, "unit": "MLUPS", "n_gpus": world, "steps": args.steps,
            "warmup": args.warmup, "ms_per_step": ms_graph, "higher_is_better": True,
            "scaling": "strong" if world > 1 else "weak",
@@ -382,10 +422,8 @@ def run_ensemble(args):
                       "parallelism": f"instances sharded over {world} ranks" if world > 1 else "single GPU"},
            "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                         "frac": achieved / peak,
-                        "kernel": (f"k_ens_step2 (two steps per launch, graph-replayed, autotuned launch {cfg})"
-                                   if args.ens_spp == 2 else "k_ens_step (persistent, graph-replayed)"),
-                        "peak_source": src},
-           "steps_per_launch": args.ens_spp, "tuner_timings": ensemble_tuner_timings(inst),
+                        "kernel": ens_kernel, "peak_source": src},
+           "steps_per_launch": ens_steps, "tuner_timings": ensemble_tuner_timings(inst),
            "one_step_graph_mlups": nodes_r0 * steps / (ms_g1 / 1e3) / 1e6,
            "persistent_grid_graph_mlups": nodes_r0 * steps / (ms_pgrid / 1e3) / 1e6,
            "persistent_no_graph_mlups": nodes_r0 * steps / (ms_pers / 1e3) / 1e6,
@@ -396,7 +434,7 @@ def run_ensemble(args):
                    "d2h_bytes_per_step": int(host_stats.numel() * host_stats.element_size()),
                    "read_back": "per-instance FP64 statistics (lbm_ensemble_reduce)",
                    "max_relative_mass_drift": mass_drift},
-           "gpu_launches": args.steps * (1 + steps // args.ens_spp)}
+           "gpu_launches": args.steps * (1 + ens_launches)}
     if clocks is not None:
         out["clocks"] = clocks
     print(json.dumps(out), flush=True)
@@ -690,7 +728,10 @@ def run_gaussian3d(args):
     torch.cuda.synchronize()
     clocks = clocks_summary(clk)
     ms = t0.elapsed_time(t1) / args.steps
-    launch_ms = statistics.mean(a.elapsed_time(b) for a, b in ev) / lbm_steps
+    # large periodic FP32 lattices: sweeps of two steps, in pairs, where the launch is left to the library
+    sweeps = prec == "f32" and args.block_rows == 0 and n ** 3 >= 1 << 22
+    launches = lbm_steps // 4 * 2 + lbm_steps % 4 if sweeps else lbm_steps
+    launch_ms = statistics.mean(a.elapsed_time(b) for a, b in ev) / launches
     cells = n ** 3
     # populations read + written (BF16S: 2 B each plus the 4 B shift plane)
     bpu = {"f64": 19 * 2 * 8, "f32": 19 * 2 * 4, "bf16s": 19 * 2 * 2 + 2 * 4}[prec]
@@ -704,10 +745,12 @@ def run_gaussian3d(args):
                                   f"{lbm_steps} steps per job", "nx": n, "ny": n, "nz": n,
                       "l2": "inputs larger than L2 (two population buffers of 0.67 to 2.5 GB each)"},
            "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
-                        "traffic": None, "kernel": "k_step3 (D3Q19 fused pull-stream + collide)",
-                        "algorithmic_bytes_per_update": bpu, "avg_launch_ms": launch_ms,
+                        "traffic": None,
+                        "kernel": ("k_sweep3 (D3Q19, two fused pull-stream + collide steps per sweep)" if sweeps
+                                   else "k_step3 (D3Q19 fused pull-stream + collide)"),
+                        "algorithmic_bytes_per_node_and_launch": bpu, "avg_launch_ms": launch_ms,
                         "peak_source": f"{src} (MEASURED_PEAKS.json hbm_gbs)" if src == "measured" else src},
-           "gre_vs_eq60": g[1] / g[2], "gpu_launches": args.steps * (1 + lbm_steps + 2)}
+           "gre_vs_eq60": g[1] / g[2], "gpu_launches": args.steps * (1 + launches + 2)}
     if clocks is not None:
         out["clocks"] = clocks
     print(json.dumps(out), flush=True)
@@ -784,7 +827,7 @@ def c3_measure(prec, cfg, lbm_steps, steps, warmup, warm_lbm_steps=None):
     clocks = clocks_summary(clk)
     ms = t0.elapsed_time(t1) / steps
     spp = cfg.get("steps_per_pass", 1)
-    launches = lbm_steps // spp + lbm_steps % spp
+    launches = step_launches(lbm_steps, prec, spp, cfg.get("kernel_variant", 0), cfg.get("block_rows", 0), n, n)
     launch_ms = statistics.mean(a.elapsed_time(b) for a, b in ev) / launches
     phi = s.phi().cpu().numpy()
     del s
@@ -806,7 +849,7 @@ def extra_c3(prec, lbm_steps, steps, warmup, fp64_phi, peak, src):
     r = c3_measure(prec, cfg, lbm_steps, steps, warmup)
     cells = p["nx"] * p["ny"]
     achieved = BYTES_PER_UPDATE[prec] * cells / (r["avg_launch_ms"] / 1e3) / 1e9
-    kernel, traffic = step_kernel(prec, cfg["steps_per_pass"], cfg["kernel_variant"])
+    kernel, traffic = step_kernel(prec, cfg["steps_per_pass"], cfg["kernel_variant"], cfg["block_rows"], p["nx"], p["ny"])
     out = {"workload": f"{WORKLOAD}, {lbm_steps} steps per job, storage {prec}", "value": r["mlups"],
            "unit": "MLUPS", "ms_per_job": r["ms_per_job"], "timed_jobs": steps, "config": cfg,
            "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
@@ -882,8 +925,8 @@ def extra_adjoint(warmup):
 
 
 def extra_ensemble(warmup, steps):
-    """Sub-record of the 256-instance ensemble (1000 steps per job): two steps
-    per launch replayed from a CUDA graph, against one launch per instance and
+    """Sub-record of the 256-instance ensemble (1000 steps per job): the autotuned
+    launch replayed from a CUDA graph, against one launch per instance and
     step (256 launches per step)."""
     import torch
 
@@ -927,7 +970,7 @@ def extra_ensemble(warmup, steps):
     return {"workload": f"ensemble_256: 256 instances, sides 64..1024 ({nodes} nodes), D(phi)=D0(1+phi), "
                         f"{lbm_steps} steps per job, FP32",
             "value": nodes * lbm_steps / (ms_graph / 1e3) / 1e6, "unit": "MLUPS",
-            "mode": "two steps per launch over the tiles of all instances, 100-step CUDA graph replayed",
+            "mode": f"100-step CUDA graph replayed, {ensemble_launches(lbm_steps, 2, cfg, inst)[1]}",
             "autotuned_launch": cfg, "tuner_timings": ensemble_tuner_timings(inst),
             "per_instance_launches_mlups": nodes * lbm_steps / (ms_sep / 1e3) / 1e6,
             "speedup_vs_256_launches_per_step": ms_sep / ms_graph, "finite": finite, "clocks": clocks}
@@ -1124,14 +1167,14 @@ def main():
     torch.cuda.empty_cache()
 
     if rank == 0:
-        launches_per_job = lbm_steps // args.spp + lbm_steps % args.spp
+        launches_per_job = step_launches(lbm_steps, args.prec, args.spp, args.variant, args.block_rows, nx, ny)
         launch_ms = statistics.mean(step_kernels_ms) / launches_per_job
         # one launch reads and writes every population once, whatever the
         # number of time steps it advances
         alg_bytes = BYTES_PER_UPDATE[args.prec] * cells
         achieved = alg_bytes / (launch_ms / 1e3) / 1e9
         peak, src = measured_peak()
-        kernel, traffic = step_kernel(args.prec, args.spp, args.variant)
+        kernel, traffic = step_kernel(args.prec, args.spp, args.variant, args.block_rows, nx, ny)
         out = {
             "metric": "MLUPS", "value": value, "unit": "MLUPS", "n_gpus": world, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": ms_per_step, "higher_is_better": True, "scaling": "weak",
