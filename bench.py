@@ -35,10 +35,10 @@ import workloads as W  # noqa: E402
 
 WORKLOAD = "aniso_dirichlet_4096"
 BYTES_PER_UPDATE = {"f32": 72, "bf16s": 44, "f64": 144}
-# FP64 path: FP64 thread instructions per node update of k_step<F64> on this workload (ncu counts per launch of
-# 16.8 M nodes: 906.0 M DADD + 335.8 M DFMA + 201.5 M DMUL = 86.0 per update); its roof is the FP64 pipe's rate,
-# measured in the same run by the DFMA probe
-FP64_INST_PER_UPDATE = 86
+# FP64 path: FP64 thread instructions per node update of k_step<F64> on this workload, counted in relax() for the
+# family without a flux, cubic diffusion and a source (every operation is written out there and the compiler may not
+# contract them); its roof is the FP64 pipe's rate, measured in the same run by the DFMA probe
+FP64_INST_PER_UPDATE = 73
 KERNEL_SRC = [os.path.join(ROOT, "paper_1603_09577_gb300", "csrc", f)
               for f in ("kernels_step.cu", "kernels_step_vec.cu", "kernels_step2.cuh", "kernels_step2_f32.cu",
                         "kernels_step2_bf16.cu", "lbm_device.cuh")]
