@@ -35,9 +35,9 @@ import workloads as W  # noqa: E402
 
 WORKLOAD = "aniso_dirichlet_4096"
 BYTES_PER_UPDATE = {"f32": 72, "bf16s": 44, "f64": 144}
-# FP64 path: FP64 thread instructions per node update of k_step<F64> on this workload, counted in relax() for the
-# family without a flux, cubic diffusion and a source (every operation is written out there and the compiler may not
-# contract them); its roof is the FP64 pipe's rate, measured in the same run by the DFMA probe
+# FP64 path: FP64 thread instructions per node update on this workload, counted in the source of relax() for the family
+# without a flux, cubic diffusion and a source (every operation is written out there and the compiler may not contract
+# them); the roof is the FP64 pipe's rate, measured in the same run by the DFMA probe
 FP64_INST_PER_UPDATE = 73
 KERNEL_SRC = [os.path.join(ROOT, "paper_1603_09577_gb300", "csrc", f)
               for f in ("kernels_step.cu", "kernels_step_vec.cu", "kernels_step2.cuh", "kernels_step2_f32.cu",
@@ -185,17 +185,16 @@ def clocks_summary(proc):
     return {"sm_mhz": statistics.median(mhz), "sm_max_mhz": maxm, "reasons": sorted(reasons), "samples": len(mhz)}
 
 
-def ensemble_launches(nsteps, spp, cfg, inst):
-    """Step launches of a captured 100-step ensemble graph replayed over nsteps steps,
-    and their kernel: with two steps per pass and the default launch large ensembles
-    advance four steps per sweep, in pairs of sweeps."""
-    cols = sum(-(-d["nx"] // 120) * 120 * d["ny"] for d in inst)
-    if (spp == 2 and not cfg.get("persistent") and not cfg.get("pair_tiles") and cols >= 4000000
-            and all(d["nx"] >= 16 and d["ny"] >= 16 for d in inst)):
-        return nsteps // 100 * (24 + 2), "k_ens_march (four steps per sweep, graph-replayed)", 4
-    if spp == 2:
-        return nsteps // 2, f"k_ens_step2 (two steps per launch, graph-replayed, autotuned launch {cfg})", 2
-    return nsteps, "k_ens_step (persistent, graph-replayed)", 1
+def ensemble_launches(e, nsteps, cfg):
+    """Step launches of the ensemble's captured 100-step graph replayed over nsteps steps,
+    and the kernel that takes most of the steps, as the library reports its route."""
+    r = e.route(100)
+    launches = nsteps // 100 * sum(r.values())
+    if r["fours"]:
+        return launches, "k_ens_march (four steps per sweep, graph-replayed)", 4
+    if r["twos"]:
+        return launches, f"k_ens_step2 (two steps per launch, graph-replayed, autotuned launch {cfg})", 2
+    return launches, "k_ens_step (persistent, graph-replayed)", 1
 
 
 def measured_peak():
@@ -219,45 +218,27 @@ def traffic_per_launch(kernel_sha, key="k_step2"):
         return None
 
 
-def takes_march(prec, variant, rows, nx, ny):
-    """Whether this launch configuration's sweeps advance four time steps (the
-    library's choice for FP32 where it is left the launch and the lattice is large)."""
-    return (prec == "f32" and (variant, rows) in ((0, 0), (5, 4)) and nx >= 128 and ny >= 64
-            and nx * ny >= 1 << 18)
-
-
-def step_launches(nsteps, prec, spp, variant, rows, nx, ny):
-    """Step-kernel launches of one lbm_step(nsteps) call (on lattices of fewer than
-    2^18 nodes, where one launch may take up to eight steps, at most these)."""
-    if not takes_march(prec, variant, rows, nx, ny):
-        return nsteps // spp + nsteps % spp
-    # sweeps of four, then of two, then single steps; with two steps per pass an even
-    # number of fours, with one as many launches, modulo 2, as steps
-    twos, one = nsteps // 2, nsteps % 2
-    four = twos // 2
-    if four & 1 != (0 if spp == 2 else twos & 1):
-        four = max(0, four - 1)
-    two = twos - 2 * four
-    if spp == 1 and (four + two) & 1:
-        two, one = two - 1, one + 2
-    return four + two + one
-
-
-def step_kernel(prec, spp, variant, rows, nx, ny):
-    """Name of the step kernel a launch configuration runs, and its DRAM bytes per
-    launch from the committed ncu capture (None when there is none or the
-    kernel's sources changed since)."""
-    if takes_march(prec, variant, rows, nx, ny):
-        return "k_march (four fused pull-stream + collide steps per sweep)", None
-    if spp == 2 and variant == 5:
-        return ("k_step2p (two fused pull-stream + collide steps per sweep, pair tiles)",
+def step_kernel(s, lbm_steps):
+    """Step-kernel launches of s.step(lbm_steps), the name of the kernel that takes most
+    of the steps (as the library reports its route) and its DRAM bytes per launch from the
+    committed ncu capture (None when there is none or the kernel's sources changed since)."""
+    r, prec, variant = s.route(lbm_steps), s.prec, s.desc.kernel_variant
+    n = sum(r.values())
+    if r["tiles"]:
+        per = -(-lbm_steps // n)
+        return n, f"k_tile (up to {per} fused pull-stream + collide step{'s' if per > 1 else ''} per launch)", None
+    if r["fours"]:
+        return n, "k_march (four fused pull-stream + collide steps per sweep)", None
+    if r["pairs"]:
+        return (n, "k_step2p (two fused pull-stream + collide steps per sweep, pair tiles)",
                 traffic_per_launch(src_sha(PAIR_SRC), f"k_step2p_{prec}"))
-    if spp == 2:
-        return ("k_step2 (two fused pull-stream + collide steps per sweep)",
-                traffic_per_launch(src_sha(KERNEL_SRC)) if prec == "f32" else None)
-    if variant == 2 or (variant == 0 and prec == "bf16s"):
-        return "k_step_v4 (fused pull-stream + collide, four nodes per thread)", None
-    return "k_step (fused pull-stream + collide)", None
+    if r["twos"]:
+        name = {3: "k_step2m", 4: "k_step2_tma"}.get(variant, "k_step2")
+        return (n, f"{name} (two fused pull-stream + collide steps per sweep)",
+                traffic_per_launch(src_sha(KERNEL_SRC)) if prec == "f32" and name == "k_step2" else None)
+    if variant == 2 or (variant == 0 and prec == "bf16s" and s.nx % 4 == 0):
+        return n, "k_step_v4 (fused pull-stream + collide, four nodes per thread)", None
+    return n, "k_step (fused pull-stream + collide)", None
 
 
 def run_reference(args):
@@ -410,7 +391,7 @@ def run_ensemble(args):
     else:
         nodes_r0 = nodes
     peak, src = measured_peak()
-    ens_launches, ens_kernel, ens_steps = ensemble_launches(steps, args.ens_spp, cfg, inst)
+    ens_launches, ens_kernel, ens_steps = ensemble_launches(e, steps, cfg)
     achieved = 72.0 * nodes_r0 * ens_launches / (ms_graph / 1e3) / 1e9
     out = {"metric": "MLUPS", "value": val, "unit": "MLUPS", "n_gpus": world, "steps": args.steps,
            "warmup": args.warmup, "ms_per_step": ms_graph, "higher_is_better": True,
@@ -728,9 +709,8 @@ def run_gaussian3d(args):
     torch.cuda.synchronize()
     clocks = clocks_summary(clk)
     ms = t0.elapsed_time(t1) / args.steps
-    # large periodic FP32 lattices: sweeps of two steps, in pairs, where the launch is left to the library
-    sweeps = prec == "f32" and args.block_rows == 0 and n ** 3 >= 1 << 22
-    launches = lbm_steps // 4 * 2 + lbm_steps % 4 if sweeps else lbm_steps
+    route = s.route(lbm_steps)
+    sweeps, launches = route["sweeps"], sum(route.values())
     launch_ms = statistics.mean(a.elapsed_time(b) for a, b in ev) / launches
     cells = n ** 3
     # populations read + written (BF16S: 2 B each plus the 4 B shift plane)
@@ -826,14 +806,13 @@ def c3_measure(prec, cfg, lbm_steps, steps, warmup, warm_lbm_steps=None):
     torch.cuda.synchronize()
     clocks = clocks_summary(clk)
     ms = t0.elapsed_time(t1) / steps
-    spp = cfg.get("steps_per_pass", 1)
-    launches = step_launches(lbm_steps, prec, spp, cfg.get("kernel_variant", 0), cfg.get("block_rows", 0), n, n)
+    launches, kernel, traffic = step_kernel(s, lbm_steps)
     launch_ms = statistics.mean(a.elapsed_time(b) for a, b in ev) / launches
     phi = s.phi().cpu().numpy()
     del s
     torch.cuda.empty_cache()
     return {"mlups": n * n * lbm_steps / (ms / 1e3) / 1e6, "ms_per_job": ms, "avg_launch_ms": launch_ms,
-            "launches_per_job": launches, "clocks": clocks, "phi": phi}
+            "launches_per_job": launches, "kernel": kernel, "traffic": traffic, "clocks": clocks, "phi": phi}
 
 
 def rel_l2(a, b):
@@ -849,11 +828,10 @@ def extra_c3(prec, lbm_steps, steps, warmup, fp64_phi, peak, src):
     r = c3_measure(prec, cfg, lbm_steps, steps, warmup)
     cells = p["nx"] * p["ny"]
     achieved = BYTES_PER_UPDATE[prec] * cells / (r["avg_launch_ms"] / 1e3) / 1e9
-    kernel, traffic = step_kernel(prec, cfg["steps_per_pass"], cfg["kernel_variant"], cfg["block_rows"], p["nx"], p["ny"])
     out = {"workload": f"{WORKLOAD}, {lbm_steps} steps per job, storage {prec}", "value": r["mlups"],
            "unit": "MLUPS", "ms_per_job": r["ms_per_job"], "timed_jobs": steps, "config": cfg,
            "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
-                        "kernel": kernel, "traffic": traffic,
+                        "kernel": r["kernel"], "traffic": r["traffic"],
                         "algorithmic_bytes_per_launch": BYTES_PER_UPDATE[prec] * cells,
                         "avg_launch_ms": r["avg_launch_ms"], "peak_source": src,
                         "one_step_roof_mlups": peak * 1e3 / BYTES_PER_UPDATE[prec]},
@@ -962,6 +940,7 @@ def extra_ensemble(warmup, steps):
         ms_graph = timed(job_graph, steps, side)
         clocks = clocks_summary(clk)
         ms_sep = timed(job_launches, max(1, steps // 2), side)
+        mode = ensemble_launches(e, lbm_steps, cfg)[1]
         out_phi = e.phi()
         finite = bool(torch.isfinite(out_phi).all())
     nodes = e.nodes
@@ -970,7 +949,7 @@ def extra_ensemble(warmup, steps):
     return {"workload": f"ensemble_256: 256 instances, sides 64..1024 ({nodes} nodes), D(phi)=D0(1+phi), "
                         f"{lbm_steps} steps per job, FP32",
             "value": nodes * lbm_steps / (ms_graph / 1e3) / 1e6, "unit": "MLUPS",
-            "mode": f"100-step CUDA graph replayed, {ensemble_launches(lbm_steps, 2, cfg, inst)[1]}",
+            "mode": f"100-step CUDA graph replayed, {mode}",
             "autotuned_launch": cfg, "tuner_timings": ensemble_tuner_timings(inst),
             "per_instance_launches_mlups": nodes * lbm_steps / (ms_sep / 1e3) / 1e6,
             "speedup_vs_256_launches_per_step": ms_sep / ms_graph, "finite": finite, "clocks": clocks}
@@ -1048,10 +1027,10 @@ def extras(args, lbm_steps, headline_phi, peak, src, fp64_rate):
     ex = {"fp64_pipe": fp64_rate}
     # FP64: one full job (about 8 s), the reference field of the other precisions
     r = c3_measure("f64", {}, lbm_steps, 1, 1, warm_lbm_steps=20)
-    ginst = FP64_INST_PER_UPDATE * cells / (r["avg_launch_ms"] / 1e3) / 1e9
+    ginst = FP64_INST_PER_UPDATE * cells * lbm_steps / (r["launches_per_job"] * r["avg_launch_ms"] / 1e3) / 1e9
     ex["fp64"] = {"workload": f"{WORKLOAD}, {lbm_steps} steps per job, storage f64", "value": r["mlups"],
                   "unit": "MLUPS", "ms_per_job": r["ms_per_job"], "timed_jobs": 1,
-                  "roofline": fp64_roofline(ginst, fp64_rate, "k_step<F64> (fused pull-stream + collide)",
+                  "roofline": fp64_roofline(ginst, fp64_rate, r["kernel"],
                                             BYTES_PER_UPDATE["f64"] * cells / (r["avg_launch_ms"] / 1e3) / 1e9 / peak,
                                             r["avg_launch_ms"]),
                   "clocks": r["clocks"]}
@@ -1163,18 +1142,17 @@ def main():
     e2e_val = whole_job_mlups(world, cells, lbm_steps, e2e_s * 1e3)
 
     headline_phi = s.phi().cpu().numpy() if (rank == 0 and world == 1 and not args.no_extras) else None
+    launches_per_job, kernel, traffic = step_kernel(s, lbm_steps)
     del s
     torch.cuda.empty_cache()
 
     if rank == 0:
-        launches_per_job = step_launches(lbm_steps, args.prec, args.spp, args.variant, args.block_rows, nx, ny)
         launch_ms = statistics.mean(step_kernels_ms) / launches_per_job
         # one launch reads and writes every population once, whatever the
         # number of time steps it advances
         alg_bytes = BYTES_PER_UPDATE[args.prec] * cells
         achieved = alg_bytes / (launch_ms / 1e3) / 1e9
         peak, src = measured_peak()
-        kernel, traffic = step_kernel(args.prec, args.spp, args.variant, args.block_rows, nx, ny)
         out = {
             "metric": "MLUPS", "value": value, "unit": "MLUPS", "n_gpus": world, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": ms_per_step, "higher_is_better": True, "scaling": "weak",

@@ -182,6 +182,12 @@ int lbm_set_phi(lbm_handle h, const void *dev_phi, int prec, void *stream);
    number is chosen so that the launches of a call are even or odd as before.) The first call on a device configures kernel
    attributes: make it before any stream capture. */
 int lbm_step(lbm_handle h, int nsteps, void *stream);
+/* The step-kernel launches of lbm_step(h, nsteps), in the order they run:
+   launches[0] over small lattices' tiles (they share their steps as evenly as
+   they can), [1] of four steps, [2] of two steps over pair tiles, [3] of two steps
+   by another kernel, [4] of one step. sms: SMs of the device to plan for; 0: the
+   current device's. Host only; needs lbm_set_coeffs. */
+int lbm_step_route(lbm_handle h, int nsteps, int sms, int launches[5]);
 
 /* Dirichlet data of the LBM_NEE axes. dev_values: device array of nrec >= 1
    records, each 2 (nx + ny) doubles laid out west[ny], east[ny], south[nx],
@@ -347,6 +353,9 @@ int lbm_ensemble_set_tiles(lbm_ensemble e, int pair_tiles);
    launch when configured, an odd remainder with one); mode 1: one launch per
    instance per step (one-step arithmetic, for comparison). */
 int lbm_ensemble_step(lbm_ensemble e, int nsteps, int mode, void *stream);
+/* The launches of that call, in the order they run: launches[0] of four steps,
+   [1] of two, [2] of one step (with mode 1 one launch per instance and step). */
+int lbm_ensemble_step_route(lbm_ensemble e, int nsteps, int mode, int launches[3]);
 /* Capture nsteps persistent steps (a positive multiple of 2 * steps per
    launch) on a non-default stream into a CUDA graph held by the ensemble;
    lbm_ensemble_replay launches it (advancing the state by nsteps). */

@@ -86,6 +86,9 @@ int lbm3_set_phi(lbm3_handle h, const void *dev_phi, int prec, void *stream);
    take an even number of sweeps of two steps (the same states bit for bit); their
    kernel's attributes are set by lbm3_set_phi, lbm3_load or the first call. */
 int lbm3_step(lbm3_handle h, int nsteps, void *stream);
+/* The launches of that call: launches[0] sweeps of two steps, then launches[1]
+   single steps. Host only. */
+int lbm3_step_route(lbm3_handle h, int nsteps, int launches[2]);
 /* Checkpoint / resume: the state is lbm3_state_bytes bytes (the 19 population
    planes and, for LBM_BF16S, the shift plane). dev_dst / dev_src: device
    buffers of that size, owned by the caller. Asynchronous on `stream`.

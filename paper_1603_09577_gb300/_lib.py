@@ -67,6 +67,7 @@ SIGNATURES = {
     "lbm_set_phi": [_VP, _VP, _I, _VP],
     "lbm_set_phi_host": [_VP, _VP, _I, _VP],
     "lbm_step": [_VP, _I, _VP],
+    "lbm_step_route": [_VP, _I, _I, ctypes.POINTER(_I)],
     "lbm_set_dirichlet": [_VP, _VP, _I],
     "lbm_get_phi": [_VP, _VP, _I, _VP],
     "lbm_get_phi_host": [_VP, _VP, _I, _VP],
@@ -91,6 +92,7 @@ SIGNATURES = {
     "lbm3_set_coeffs": [_VP, ctypes.POINTER(Coeffs3)],
     "lbm3_set_phi": [_VP, _VP, _I, _VP],
     "lbm3_step": [_VP, _I, _VP],
+    "lbm3_step_route": [_VP, _I, ctypes.POINTER(_I)],
     "lbm3_get_phi": [_VP, _VP, _I, _VP],
     "lbm3_state_bytes": [_VP, ctypes.POINTER(_SZ)],
     "lbm3_save": [_VP, _VP, _VP],
@@ -103,6 +105,7 @@ SIGNATURES = {
     "lbm_ensemble_info": [_VP, ctypes.POINTER(ctypes.c_longlong), ctypes.POINTER(_I), ctypes.POINTER(_I)],
     "lbm_ensemble_set_phi": [_VP, _VP, _I, _VP],
     "lbm_ensemble_step": [_VP, _I, _I, _VP],
+    "lbm_ensemble_step_route": [_VP, _I, _I, ctypes.POINTER(_I)],
     "lbm_ensemble_capture": [_VP, _I, _VP],
     "lbm_ensemble_configure": [_VP, _I],
     "lbm_ensemble_set_persistent": [_VP, _I],

@@ -314,6 +314,18 @@ int lbm_ensemble_step(lbm_ensemble e, int nsteps, int mode, void *stream)
     return LBM_OK;
 }
 
+int lbm_ensemble_step_route(lbm_ensemble e, int nsteps, int mode, int launches[3])
+{
+    if (!e) return fail(LBM_EINVAL, "null ensemble");
+    if (!launches) return fail(LBM_EINVAL, "null launch counts");
+    if (nsteps < 0) return fail(LBM_EINVAL, "negative step count");
+    if (mode != 0 && mode != 1) return fail(LBM_EINVAL, "mode must be 0 (persistent) or 1 (one launch per instance)");
+    launches[0] = fours(e, mode, nsteps);
+    launches[1] = mode == 0 && e->spp == 2 ? (nsteps - 4 * launches[0]) / 2 : 0;
+    launches[2] = (nsteps - 4 * launches[0] - 2 * launches[1]) * (mode == 0 ? 1 : e->count);
+    return LBM_OK;
+}
+
 int lbm_ensemble_configure(lbm_ensemble e, int steps_per_pass)
 {
     if (!e) return fail(LBM_EINVAL, "null ensemble");

@@ -528,22 +528,30 @@ int lbm3_step(lbm3_handle h, int nsteps, void *stream)
     if (int rc = ready3(h)) return rc;
     if (!h->phi_set) return fail(LBM_EINVAL, "lbm3_set_phi has not been called");
     if (nsteps < 0) return fail(LBM_EINVAL, "negative step count");
-    int i = 0;
-    if (sweep3_wanted(h)) {
-        // an even number of two-step sweeps, so that the launches of a call stay even or odd
-        // in number as its steps (a captured call ends on the buffer it started from)
+    // an even number of two-step sweeps, so that the launches of a call stay even or odd
+    // in number as its steps (a captured call ends on the buffer it started from)
+    int launches[2];
+    if (int rc = lbm3_step_route(h, nsteps, launches)) return rc;
+    if (launches[0])
         if (int rc = cuda_check(launch_sweep3(h, true, (cudaStream_t)stream), "lbm3_step (kernel attributes)")) return rc;
-        for (; i + 4 <= nsteps; i += 4)
-            for (int j = 0; j < 2; ++j) {
-                if (int rc = cuda_check(launch_sweep3(h, false, (cudaStream_t)stream), "lbm3_step (two steps per sweep)"))
-                    return rc;
-                h->cur ^= 1;
-            }
+    for (int i = 0; i < launches[0]; ++i) {
+        if (int rc = cuda_check(launch_sweep3(h, false, (cudaStream_t)stream), "lbm3_step (two steps per sweep)")) return rc;
+        h->cur ^= 1;
     }
-    for (; i < nsteps; ++i) {
+    for (int i = 0; i < launches[1]; ++i) {
         if (int rc = cuda_check(launch3(h, nullptr, 0, (cudaStream_t)stream), "lbm3_step")) return rc;
         h->cur ^= 1;
     }
+    return LBM_OK;
+}
+
+int lbm3_step_route(lbm3_handle h, int nsteps, int launches[2])
+{
+    if (!h) return fail(LBM_EINVAL, "null handle");
+    if (!launches) return fail(LBM_EINVAL, "null launch counts");
+    if (nsteps < 0) return fail(LBM_EINVAL, "negative step count");
+    launches[0] = sweep3_wanted(h) ? nsteps / 4 * 2 : 0;
+    launches[1] = nsteps - 2 * launches[0];
     return LBM_OK;
 }
 

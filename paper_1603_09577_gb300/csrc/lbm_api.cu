@@ -243,12 +243,12 @@ static cudaError_t launch_tile(const lbm_solver *s, int src, int steps, bool pre
 // 4.14 at 400^2 (tiles 2.18), 4.17 at 600^2 (4.00), 5.74 at 803 x 797 (7.00). FP64, the
 // one-step kernel, whose blocks of 256 nodes take two turns of an SM's FP64 pipe
 // each: 8.28 at 128^2 (tiles 5.21), 14.4 at 200^2 (9.31), 19.0 at 301^2 (16.9).
-static bool tile_wanted(const lbm_solver *s)
+static bool tile_wanted(const lbm_solver *s, int sms)
 {
     const double n = (double)s->d.nx * s->d.ny;
     if (s->d.prec == LBM_F64) {
         const long long blocks = (long long)((s->d.nx + 31) / 32) * ((s->d.ny + 7) / 8);
-        return s->plan.us < 3.2 + 5.2 * (double)((blocks + s->sms - 1) / s->sms);
+        return s->plan.us < 3.2 + 5.2 * (double)((blocks + sms - 1) / sms);
     }
     return s->plan.us < std::max(4.1, 2.5 + n / 210e3);
 }
@@ -289,11 +289,11 @@ static int tile_launches(const lbm_solver *s, int nsteps)
 // step per pass 60^2 4.4 -> 2.0, 301^2 6.4 -> 4.1, 500^2 8.5 -> 7.0, 700^2 10.6 -> 12.7; two
 // 6.4 -> 1.9, 6.4 -> 4.1, 7.7 -> 7.0, 9.8 -> 12.7; FP64 60^2 24.9 -> 11.1, 200^2 45.4 -> 28.1,
 // 500^2 103 -> 97, 700^2 174 -> 165 (there with one step per launch: smaller blocks).
-static bool tile_general_wanted(lbm_solver *s)
+static bool tile_general_wanted(lbm_solver *s, int sms)
 {
     if (s->d.kernel_variant != 0 || s->d.block_rows != 0 || s->c.cfree || s->d.prec == LBM_BF16S || s->c.conv > 2) return false;
     if ((long long)s->d.nx * s->d.ny > (s->d.prec == LBM_F64 ? 500000 : 250000)) return false;
-    if (s->plan.T == 0) s->plan = tile_plan(s->d.nx, s->d.ny, s->d.prec == LBM_F64, true, s->sms);
+    if (s->plan.T == 0) s->plan = tile_plan(s->d.nx, s->d.ny, s->d.prec == LBM_F64, true, sms);
     return s->plan.us < 1e29 && (s->d.prec == LBM_F64 || s->plan.T >= 2);
 }
 
@@ -308,55 +308,56 @@ static cudaError_t launch_tile_general(const lbm_solver *s, int src, const doubl
              : launch_tile_general_f32_b(s, src, records, steps, prepare, st);
 }
 
-// nsteps as sweeps of four, two and one steps. The number of launches stays odd or
-// even as it is with steps_per_pass steps each (n, or n/2 + n%2), so that a
-// captured call that ended on the buffer it started from still does: with m pairs
-// of steps, sweeps of four are even in number (two steps per pass) or as m (one).
-static int step_auto(lbm_handle h, int nsteps, cudaStream_t st)
+// The launches of a call, in the order they run
+struct Route {
+    int tiles = 0;      // small lattices' tiles, which share their steps as evenly as they can
+    int fours = 0;      // sweeps of four steps (the marching kernel)
+    int pairs = 0;      // sweeps of two steps over pair tiles
+    int twos = 0;       // sweeps of two steps by another kernel (the one that the descriptor names)
+    int ones = 0;       // single steps
+};
+
+// The route of nsteps steps on a device of `sms` SMs. On the path left to the library
+// the number of launches stays odd or even as it is with steps_per_pass steps each (n,
+// or n/2 + n%2), so that a captured call that ended on the buffer it started from
+// still does: with m pairs of steps, sweeps of four are even in number (two steps per
+// pass) or as m (one).
+static Route plan_route(lbm_solver *h, int nsteps, int sms)
 {
-    if (int rc = device_sms(h)) return rc;
-    if (h->plan.T == 0) h->plan = tile_plan(h->d.nx, h->d.ny, h->d.prec == LBM_F64, false, h->sms);
-    if (tile_wanted(h)) {
-        if (int rc = cuda_check(launch_tile(h, h->cur, 1, true, st), "lbm_step (kernel attributes)")) return rc;
-        const int launches = tile_launches(h, nsteps);
-        for (int i = 0, done = 0; i < launches; ++i) {
-            const int steps = (nsteps - done) / (launches - i) + ((nsteps - done) % (launches - i) != 0);
-            if (int rc = cuda_check(launch_tile(h, h->cur, steps, false, st), "lbm_step (small lattice)")) return rc;
-            h->cur ^= 1;
-            h->t += steps;
-            done += steps;
+    Route r;
+    if (general_path(h)) {
+        if (tile_general_wanted(h, sms)) r.tiles = tile_launches(h, nsteps);
+        else if (h->d.steps_per_pass == 2) { r.twos = nsteps / 2; r.ones = nsteps % 2; }
+        else r.ones = nsteps;
+        return r;
+    }
+    if (!auto_path(h)) {
+        if (h->d.steps_per_pass == 2) {
+            (h->d.kernel_variant == 5 ? r.pairs : r.twos) = nsteps / 2;
+            r.ones = nsteps % 2;
+        } else {
+            r.ones = nsteps;
         }
-        return LBM_OK;
+        return r;
     }
-    const int m = h->d.prec == LBM_F64 ? 0 : nsteps / 2, one = nsteps - 2 * m;
-    int four = 0;
+    if (h->plan.T == 0) h->plan = tile_plan(h->d.nx, h->d.ny, h->d.prec == LBM_F64, false, sms);
+    if (tile_wanted(h, sms)) {
+        r.tiles = tile_launches(h, nsteps);
+        return r;
+    }
+    const int m = h->d.prec == LBM_F64 ? 0 : nsteps / 2;
     if (h->d.prec == LBM_F32 && march_wanted(h)) {
-        if (int rc = cuda_check(launch_march(h, h->cur, true, st), "lbm_step (kernel attributes)")) return rc;
-        four = m / 2;
-        if ((four & 1) != (h->d.steps_per_pass == 2 ? 0 : (m & 1))) --four;
-        if (four < 0) four = 0;
+        r.fours = m / 2;
+        if ((r.fours & 1) != (h->d.steps_per_pass == 2 ? 0 : (m & 1))) --r.fours;
+        if (r.fours < 0) r.fours = 0;
     }
-    int two = m - 2 * four, single = one;
-    if (h->d.steps_per_pass == 1 && ((four + two) & 1)) {     // no sweeps of four to make the count even
-        --two;
-        single += 2;
+    r.pairs = m - 2 * r.fours;
+    r.ones = nsteps - 2 * m;
+    if (h->d.steps_per_pass == 1 && ((r.fours + r.pairs) & 1)) {     // no sweeps of four to make the count even
+        --r.pairs;
+        r.ones += 2;
     }
-    for (int i = 0; i < four; ++i) {
-        if (int rc = cuda_check(launch_march(h, h->cur, false, st), "lbm_step (four steps per sweep)")) return rc;
-        h->cur ^= 1;
-        h->t += 4;
-    }
-    for (int i = 0; i < two; ++i) {
-        if (int rc = cuda_check(launch_step2p_f32(h, h->cur, st), "lbm_step (two steps per sweep)")) return rc;
-        h->cur ^= 1;
-        h->t += 2;
-    }
-    for (int i = 0; i < single; ++i) {
-        if (int rc = cuda_check(launch_step(h, h->cur, st), "lbm_step")) return rc;
-        h->cur ^= 1;
-        h->t += 1;
-    }
-    return LBM_OK;
+    return r;
 }
 
 static int check_handle(lbm_handle h)
@@ -555,73 +556,77 @@ int lbm_step(lbm_handle h, int nsteps, void *stream)
     if (!h->phi_set) return fail(LBM_EINVAL, "lbm_set_phi has not been called");
     if (nsteps < 0) return fail(LBM_EINVAL, "negative step count");
     cudaStream_t st = (cudaStream_t)stream;
+    const bool general = general_path(h), nee = is_nee(h);
+    if (nee && !h->dir_vals) return fail(LBM_EINVAL, "lbm_set_dirichlet has not been called");
+    // the general kernels pick the record from the device count of steps since the
+    // records were set plus the sweep's place in this call (dir_off); one
+    // one-thread launch advances the count after the call's sweeps
+    const double *records = nee ? h->dir_vals : nullptr;
+    if (nee)
+        if (int rc = flush_record_reset(h, st)) return rc;
+    if (int rc = device_sms(h)) return rc;
+    const Route r = plan_route(h, nsteps, h->sms);
+    if (r.tiles || r.fours)
+        if (int rc = cuda_check(!r.tiles   ? launch_march(h, h->cur, true, st)
+                                : general ? launch_tile_general(h, h->cur, records, 1, true, st)
+                                          : launch_tile(h, h->cur, 1, true, st), "lbm_step (kernel attributes)"))
+            return rc;
     int done = 0;
-    if (general_path(h)) {
-        const bool nee = is_nee(h);
-        if (nee && !h->dir_vals) return fail(LBM_EINVAL, "lbm_set_dirichlet has not been called");
-        // the kernels pick the record from the device count of steps since the
-        // records were set plus the sweep's place in this call (dir_off); one
-        // one-thread launch advances the count after the call's sweeps
-        const double *records = nee ? h->dir_vals : nullptr;
-        if (nee)
-            if (int rc = flush_record_reset(h, st)) return rc;
-        if (int rc = device_sms(h)) return rc;
-        if (tile_general_wanted(h)) {
-            if (int rc = cuda_check(launch_tile_general(h, h->cur, records, 1, true, st), "lbm_step (kernel attributes)"))
-                return rc;
-            const int launches = tile_launches(h, nsteps);
-            for (int i = 0; i < launches; ++i) {
-                const int left = launches - i, steps = (nsteps - done + left - 1) / left;
-                h->dir_off = done;
-                if (int rc = cuda_check(launch_tile_general(h, h->cur, records, steps, false, st),
-                                        "lbm_step (general, small lattice)"))
-                    return rc;
-                h->cur ^= 1;
-                h->t += steps;
-                done += steps;
-            }
-        }
-        if (h->d.steps_per_pass == 2) {
-            for (; done + 2 <= nsteps; done += 2) {
-                h->dir_off = done;
-                if (int rc = cuda_check(launch_step2_general(h, h->cur, records, st),
-                                        "lbm_step (general, two steps per pass)"))
-                    return rc;
-                h->cur ^= 1;
-                h->t += 2;
-            }
-        }
-        for (; done < nsteps; ++done) {
-            h->dir_off = done;
-            if (int rc = cuda_check(launch_general(h, h->cur, records, nullptr, 0, st), "lbm_step (general)"))
-                return rc;
-            h->cur ^= 1;
-            h->t += 1;
-        }
-        h->dir_off = 0;
-        if (nee && h->dir_nrec > 1 && nsteps > 0)
-            if (int rc = cuda_check(launch_tick(h->dir_counter, nsteps, st), "lbm_step (records)")) return rc;
-        return LBM_OK;
-    }
-    if (auto_path(h)) return step_auto(h, nsteps, st);
-    if (h->d.steps_per_pass == 2) {
-        for (; done + 2 <= nsteps; done += 2) {
-            const cudaError_t e = h->d.kernel_variant == 3   ? launch_step2m(h, h->cur, st)
-                                  : h->d.kernel_variant == 4 ? launch_step2_tma(h, h->cur, st)
-                                  : h->d.kernel_variant == 5 ? (h->d.prec == LBM_F32 ? launch_step2p_f32(h, h->cur, st)
-                                                                                     : launch_step2p_bf16s(h, h->cur, st))
-                                                             : launch_step2(h, h->cur, st);
-            if (int rc = cuda_check(e, "lbm_step (two steps per pass)")) return rc;
-            h->cur ^= 1;
-            h->t += 2;
-        }
-    }
-    const bool vec = h->d.kernel_variant == 2 || (h->d.kernel_variant == 0 && step_v4_preferred(h));
-    for (; done < nsteps; ++done) {
-        if (int rc = cuda_check(vec ? launch_step_v4(h, h->cur, st) : launch_step(h, h->cur, st), "lbm_step")) return rc;
+    auto advance = [&](cudaError_t e, int steps, const char *what) {
+        if (int rc = cuda_check(e, what)) return rc;
         h->cur ^= 1;
-        h->t += 1;
+        h->t += steps;
+        done += steps;
+        h->dir_off = done;
+        return (int)LBM_OK;
+    };
+    h->dir_off = 0;
+    for (int left = r.tiles; left > 0; --left) {
+        const int steps = (nsteps - done + left - 1) / left;
+        if (int rc = advance(general ? launch_tile_general(h, h->cur, records, steps, false, st)
+                                     : launch_tile(h, h->cur, steps, false, st), steps, "lbm_step (small lattice)"))
+            return rc;
     }
+    for (int i = 0; i < r.fours; ++i)
+        if (int rc = advance(launch_march(h, h->cur, false, st), 4, "lbm_step (four steps per sweep)")) return rc;
+    for (int i = 0; i < r.pairs; ++i)
+        if (int rc = advance(h->d.prec == LBM_BF16S ? launch_step2p_bf16s(h, h->cur, st) : launch_step2p_f32(h, h->cur, st),
+                             2, "lbm_step (two steps per sweep)"))
+            return rc;
+    for (int i = 0; i < r.twos; ++i)
+        if (int rc = advance(general                    ? launch_step2_general(h, h->cur, records, st)
+                             : h->d.kernel_variant == 3 ? launch_step2m(h, h->cur, st)
+                             : h->d.kernel_variant == 4 ? launch_step2_tma(h, h->cur, st)
+                                                        : launch_step2(h, h->cur, st), 2, "lbm_step (two steps per pass)"))
+            return rc;
+    const bool vec = h->d.kernel_variant == 2 || (h->d.kernel_variant == 0 && step_v4_preferred(h));
+    for (int i = 0; i < r.ones; ++i)
+        if (int rc = advance(general ? launch_general(h, h->cur, records, nullptr, 0, st)
+                             : vec   ? launch_step_v4(h, h->cur, st)
+                                     : launch_step(h, h->cur, st), 1, "lbm_step"))
+            return rc;
+    h->dir_off = 0;
+    if (nee && h->dir_nrec > 1 && nsteps > 0)
+        if (int rc = cuda_check(launch_tick(h->dir_counter, nsteps, st), "lbm_step (records)")) return rc;
+    return LBM_OK;
+}
+
+int lbm_step_route(lbm_handle h, int nsteps, int sms, int launches[5])
+{
+    if (check_handle(h)) return LBM_EINVAL;
+    if (!h->coeffs_set) return fail(LBM_EINVAL, "lbm_set_coeffs has not been called");
+    if (!launches) return fail(LBM_EINVAL, "null launch counts");
+    if (nsteps < 0 || sms < 0) return fail(LBM_EINVAL, "negative step or SM count");
+    if (sms == 0) {
+        if (int rc = device_sms(h)) return rc;
+        sms = h->sms;
+    }
+    const TilePlan kept = h->plan;       // the handle's own plan is for its device's SMs
+    if (sms != h->sms) h->plan.T = 0;
+    const Route r = plan_route(h, nsteps, sms);
+    if (sms != h->sms) h->plan = kept;
+    const int n[5] = {r.tiles, r.fours, r.pairs, r.twos, r.ones};
+    for (int i = 0; i < 5; ++i) launches[i] = n[i];
     return LBM_OK;
 }
 

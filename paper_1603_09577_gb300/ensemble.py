@@ -75,6 +75,12 @@ class Ensemble:
         C.check(self.lib.lbm_ensemble_step(self.h, int(n), int(mode), _stream(stream)))
         return self
 
+    def route(self, n: int, mode: int = 0) -> dict:
+        """Launches of step(n, mode), by their number of steps (lbm_ensemble_step_route)."""
+        v = (ctypes.c_int * 3)()
+        C.check(self.lib.lbm_ensemble_step_route(self.h, int(n), int(mode), v))
+        return dict(zip(("fours", "twos", "ones"), v))
+
     def capture(self, n: int, stream=None):
         C.check(self.lib.lbm_ensemble_capture(self.h, int(n), _stream(stream)))
         return self

@@ -12,6 +12,7 @@ from . import _lib as C
 BC = {"periodic": C.LBM_PERIODIC, "abb": C.LBM_ABB, "nee": C.LBM_NEE,
       0: C.LBM_PERIODIC, 1: C.LBM_ABB, 2: C.LBM_NEE}
 SCHEME = {"B": C.LBM_SCHEME_B, "A": C.LBM_SCHEME_A}
+ROUTE_KEYS = ("tiles", "fours", "pairs", "twos", "ones")
 REDUCE_KEYS = ("sum", "abs_err", "abs_ref", "sq_err", "sq_ref", "max_abs", "nonfinite", "sum_sq")
 
 
@@ -129,6 +130,12 @@ class Solver:
     def step(self, n: int = 1, stream=None):
         C.check(self.lib.lbm_step(self.h, int(n), _stream(stream)))
         return self
+
+    def route(self, n: int, sms: int = 0) -> dict:
+        """Step-kernel launches of step(n), by kernel (lbm_step_route)."""
+        v = (ctypes.c_int * 5)()
+        C.check(self.lib.lbm_step_route(self.h, int(n), int(sms), v))
+        return dict(zip(ROUTE_KEYS, v))
 
     # -- CUDA graphs -------------------------------------------------------------
     def capture(self, nsteps: int):

@@ -61,6 +61,12 @@ class Solver3:
         C.check(self.lib.lbm3_step(self.h, int(n), _stream(stream)))
         return self
 
+    def route(self, n: int) -> dict:
+        """Launches of step(n): two-step sweeps and single steps (lbm3_step_route)."""
+        v = (ctypes.c_int * 2)()
+        C.check(self.lib.lbm3_step_route(self.h, int(n), v))
+        return dict(sweeps=v[0], ones=v[1])
+
     # -- checkpoint / resume -------------------------------------------------------
     def state_bytes(self) -> int:
         n = ctypes.c_size_t()

@@ -1,0 +1,114 @@
+"""Which kernels serve a call, asked of the library on the CPU (lbm_step_route,
+lbm3_step_route): every route adds up to the steps asked for, keeps the number of
+launches odd or even as steps_per_pass has it (captured calls then end on the buffer
+they started from), and is what the benchmark's records name."""
+import ctypes
+
+import pytest
+
+import bench
+from paper_1603_09577_gb300 import _lib as C
+from paper_1603_09577_gb300.solver import BC, ROUTE_KEYS, SCHEME
+
+SMS = (148, 152)
+
+
+class Lattice:
+    """A handle on a host stand-in for the workspace: routes need no device."""
+
+    def __init__(self, nx, ny, prec="f32", bc=("periodic", "periodic"), steps_per_pass=1, per_cell_K=False,
+                 kernel_variant=0, block_rows=0, scheme="B", conv=0, u=(0.05, 0.02), diff=0, power=1, b=0.0, r1=0.0):
+        self.lib, self.nx, self.ny, self.prec = C.lib(), nx, ny, prec
+        d = C.Desc()
+        d.nx, d.ny, d.prec, d.bc_x, d.bc_y = nx, ny, C.PREC[prec], BC[bc[0]], BC[bc[1]]
+        d.steps_per_pass, d.per_cell_K = steps_per_pass, int(per_cell_K)
+        d.kernel_variant, d.block_rows, d.scheme = kernel_variant, block_rows, SCHEME[scheme]
+        self.desc = d
+        n = ctypes.c_size_t()
+        C.check(self.lib.lbm_workspace_size(ctypes.byref(d), ctypes.byref(n)))
+        self.h = ctypes.c_void_p()
+        # the address is only recorded: nothing below touches the workspace
+        C.check(self.lib.lbm_create(ctypes.byref(self.h), ctypes.byref(d), ctypes.c_void_p(1 << 20), n.value))
+        self.set_coeffs(conv=conv, u=u, diff=diff, power=power, b=b, r1=r1, src_family=int(b != 0.0))
+
+    def set_coeffs(self, conv=0, u=(0.05, 0.02), diff=0, power=1, b=0.0, r1=0.0, src_family=0):
+        c = C.Coeffs()
+        c.conv, c.diff, c.power, c.b, c.r1, c.src_family = conv, diff, power, b, r1, src_family
+        c.u[:], c.K[:] = u, (0.02, 0.004, 0.015)
+        c.s[:] = (1.0, 1.2, 1.2, 0.0, 1.0, 0.0, 1.0, 1.1, 1.1)
+        c.Dm[:] = (1.0, 0.0, 1.0)
+        C.check(self.lib.lbm_set_coeffs(self.h, ctypes.byref(c)))
+
+    def route(self, n, sms=152):
+        v = (ctypes.c_int * 5)()
+        C.check(self.lib.lbm_step_route(self.h, n, sms, v))
+        return dict(zip(ROUTE_KEYS, v))
+
+    def __del__(self):
+        if getattr(self, "h", None):
+            self.lib.lbm_destroy(self.h)
+
+
+SIZES = [(2, 2), (64, 64), (128, 128), (400, 400), (512, 512), (600, 600), (700, 1000), (1023, 777), (64, 16384),
+         (2, 300000), (300000, 5), (128, 16384), (121, 20000), (130, 32768), (4096, 64), (2048, 2048), (4096, 4096)]
+KINDS = [dict(prec="f64"), dict(prec="f32"), dict(prec="f32", steps_per_pass=2),
+         dict(prec="f32", steps_per_pass=2, kernel_variant=5, block_rows=4), dict(prec="f32", kernel_variant=1),
+         dict(prec="f32", per_cell_K=True), dict(prec="f32", per_cell_K=True, steps_per_pass=2), dict(prec="bf16s"),
+         dict(prec="bf16s", steps_per_pass=2, kernel_variant=5, block_rows=4),
+         dict(prec="f32", scheme="A", bc=("nee", "nee"), conv=2, b=0.02),
+         dict(prec="f64", scheme="A", conv=2, b=0.02), dict(prec="f32", diff=3, steps_per_pass=2)]
+
+
+@pytest.mark.parametrize("kind", KINDS, ids=lambda k: "-".join(f"{a}={b}" for a, b in k.items()))
+@pytest.mark.parametrize("walls", [False, True])
+def test_routes_add_up_and_keep_the_parity(kind, walls):
+    for nx, ny in SIZES:
+        kw = dict(kind)
+        if "nee" in kw.get("bc", ()) and min(nx, ny) < 3:
+            continue
+        if walls and "bc" not in kw:
+            kw["bc"] = ("abb", "abb")
+        s = Lattice(nx, ny, **kw)
+        spp = kw.get("steps_per_pass", 1)
+        for sms in SMS:
+            for n in (0, 1, 2, 3, 4, 5, 6, 7, 8, 12, 20, 23, 100):
+                r = s.route(n, sms)
+                assert min(r.values()) >= 0, (nx, ny, n, r)
+                fixed = 4 * r["fours"] + 2 * (r["pairs"] + r["twos"]) + r["ones"]
+                if r["tiles"]:
+                    assert fixed == 0 and r["tiles"] <= n, (nx, ny, n, r)
+                else:
+                    assert fixed == n, (nx, ny, n, r)
+                wanted = n // 2 + n % 2 if spp == 2 else n
+                assert sum(r.values()) % 2 == wanted % 2, (nx, ny, n, r)
+
+
+def test_the_benchmark_names_the_kernel_that_runs():
+    def name(*a, steps=100, **kw):
+        n, kernel, _ = bench.step_kernel(Lattice152(*a, **kw), steps)
+        assert n == sum(Lattice(*a, **kw).route(steps).values())
+        return kernel.split()[0]
+
+    class Lattice152(Lattice):
+        def route(self, n, sms=152):
+            return super().route(n, sms)
+
+    assert name(512, 512) == "k_tile"
+    assert name(512, 512, per_cell_K=True) == "k_step"
+    assert name(4096, 4096, prec="f64") == "k_tile"
+    assert name(4096, 4096) == "k_march"
+    assert name(4096, 4096, prec="bf16s", steps_per_pass=2, kernel_variant=5, block_rows=4) == "k_step2p"
+    assert name(4096, 4096, prec="bf16s") == "k_step_v4"
+    assert name(1002, 517, prec="bf16s") == "k_step"
+
+
+def test_route_arguments_are_checked():
+    s = Lattice(64, 64)
+    v = (ctypes.c_int * 5)()
+    assert s.lib.lbm_step_route(None, 1, 152, v) == C.LBM_EINVAL
+    assert s.lib.lbm_step_route(s.h, -1, 152, v) == C.LBM_EINVAL
+    assert s.lib.lbm_step_route(s.h, 1, -1, v) == C.LBM_EINVAL
+    assert s.lib.lbm_step_route(s.h, 1, 152, None) == C.LBM_EINVAL
+    v2, v3 = (ctypes.c_int * 2)(), (ctypes.c_int * 3)()
+    assert s.lib.lbm3_step_route(None, 1, v2) == C.LBM_EINVAL
+    assert s.lib.lbm_ensemble_step_route(None, 1, 0, v3) == C.LBM_EINVAL
