@@ -98,7 +98,8 @@ typedef struct {
                                steps_per_pass 2 (LBM_F32 / LBM_BF16S), the tile
                                kernel with two x-adjacent nodes per thread and
                                paired (vector) loads and stores; with block_rows
-                               4 and LBM_F32 as 0, automatic                  */
+                               4 and LBM_F32 as 0, automatic (exactly these tiles
+                               with lbm_set_launch_fixed)                         */
     int block_rows;         /* rows of 32-thread warps per thread block: 0 (= 8),
                                1, 2, 4 or 8; for kernel_variant 3 the rows each
                                warp marches are 16 * block_rows (0: 64); for the
@@ -182,6 +183,12 @@ int lbm_set_phi(lbm_handle h, const void *dev_phi, int prec, void *stream);
    number is chosen so that the launches of a call are even or odd as before.) The first call on a device configures kernel
    attributes: make it before any stream capture. */
 int lbm_step(lbm_handle h, int nsteps, void *stream);
+/* fixed = 1: later calls run the kernels that kernel_variant, block_rows and
+   steps_per_pass name, also where these leave the launch to the library (0: one
+   node per thread, or the 30 x 62 tiles with steps_per_pass 2; 5 with block_rows 4:
+   the 62 x 14 pair tiles). 0 (default): as described at lbm_desc. Host only; a
+   captured graph keeps the launches it was captured with. */
+int lbm_set_launch_fixed(lbm_handle h, int fixed);
 /* The step-kernel launches of lbm_step(h, nsteps), in the order they run:
    launches[0] over small lattices' tiles (they share their steps as evenly as
    they can), [1] of four steps, [2] of two steps over pair tiles, [3] of two steps

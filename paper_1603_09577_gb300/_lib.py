@@ -67,6 +67,7 @@ SIGNATURES = {
     "lbm_set_phi": [_VP, _VP, _I, _VP],
     "lbm_set_phi_host": [_VP, _VP, _I, _VP],
     "lbm_step": [_VP, _I, _VP],
+    "lbm_set_launch_fixed": [_VP, _I],
     "lbm_step_route": [_VP, _I, _I, ctypes.POINTER(_I)],
     "lbm_set_dirichlet": [_VP, _VP, _I],
     "lbm_get_phi": [_VP, _VP, _I, _VP],

@@ -224,6 +224,7 @@ static cudaError_t launch_general(const lbm_solver *s, int src, const double *bv
 // one-step kernel differ in the last bit, so that one step per pass stays one there.
 static bool auto_path(const lbm_solver *s)
 {
+    if (s->fixed) return false;
     if (s->d.prec == LBM_F64) return s->d.kernel_variant == 0 && s->d.block_rows == 0;
     return s->d.prec == LBM_F32 && !(s->d.per_cell_K && s->d.steps_per_pass == 1) &&
            ((s->d.kernel_variant == 0 && s->d.block_rows == 0) || (s->d.kernel_variant == 5 && s->d.block_rows == 4));
@@ -291,7 +292,7 @@ static int tile_launches(const lbm_solver *s, int nsteps)
 // 500^2 103 -> 97, 700^2 174 -> 165 (there with one step per launch: smaller blocks).
 static bool tile_general_wanted(lbm_solver *s, int sms)
 {
-    if (s->d.kernel_variant != 0 || s->d.block_rows != 0 || s->c.cfree || s->d.prec == LBM_BF16S || s->c.conv > 2) return false;
+    if (s->fixed || s->d.kernel_variant != 0 || s->d.block_rows != 0 || s->c.cfree || s->d.prec == LBM_BF16S || s->c.conv > 2) return false;
     if ((long long)s->d.nx * s->d.ny > (s->d.prec == LBM_F64 ? 500000 : 250000)) return false;
     if (s->plan.T == 0) s->plan = tile_plan(s->d.nx, s->d.ny, s->d.prec == LBM_F64, true, sms);
     return s->plan.us < 1e29 && (s->d.prec == LBM_F64 || s->plan.T >= 2);
@@ -608,6 +609,14 @@ int lbm_step(lbm_handle h, int nsteps, void *stream)
     h->dir_off = 0;
     if (nee && h->dir_nrec > 1 && nsteps > 0)
         if (int rc = cuda_check(launch_tick(h->dir_counter, nsteps, st), "lbm_step (records)")) return rc;
+    return LBM_OK;
+}
+
+int lbm_set_launch_fixed(lbm_handle h, int fixed)
+{
+    if (check_handle(h)) return LBM_EINVAL;
+    if (fixed != 0 && fixed != 1) return fail(LBM_EINVAL, "fixed must be 0 or 1");
+    h->fixed = fixed;
     return LBM_OK;
 }
 

@@ -39,12 +39,14 @@ class Solver:
     prec: "f64", "f32" or "bf16s"; bc: (x, y) boundary kinds "periodic", "abb"
     (anti-bounce-back walls with the constant phi_wall values: west, east, south,
     north) or "nee" (extrapolated Dirichlet nodes, values from set_dirichlet);
-    scheme: "B" (Eq. 34) or "A" (Remark II).
+    scheme: "B" (Eq. 34) or "A" (Remark II). fixed_launch: exactly the kernels that
+    kernel_variant, block_rows and steps_per_pass name (lbm_set_launch_fixed).
     """
 
     def __init__(self, nx: int, ny: int, prec: str = "f32", bc=("periodic", "periodic"),
                  phi_wall=(0.0, 0.0, 0.0, 0.0), steps_per_pass: int = 1, per_cell_K: bool = False,
-                 kernel_variant: int = 0, block_rows: int = 0, scheme: str = "B", device=None):
+                 kernel_variant: int = 0, block_rows: int = 0, scheme: str = "B", device=None,
+                 fixed_launch: bool = False):
         self.lib = C.lib()
         self.nx, self.ny, self.prec = int(nx), int(ny), prec
         self.device = torch.device(device if device is not None else "cuda")
@@ -63,6 +65,8 @@ class Solver:
         self.workspace = torch.empty(size.value, dtype=torch.uint8, device=self.device)
         self.h = ctypes.c_void_p()
         C.check(self.lib.lbm_create(ctypes.byref(self.h), ctypes.byref(d), _ptr(self.workspace), size.value))
+        if fixed_launch:
+            C.check(self.lib.lbm_set_launch_fixed(self.h, 1))
         self._out = torch.zeros(8, dtype=torch.float64, device=self.device)
 
     def __del__(self):

@@ -102,9 +102,22 @@ def test_the_benchmark_names_the_kernel_that_runs():
     assert name(1002, 517, prec="bf16s") == "k_step"
 
 
+@pytest.mark.parametrize("nx,ny", SIZES)
+def test_a_fixed_launch_runs_what_the_descriptor_names(nx, ny):
+    named = [(dict(steps_per_pass=2, kernel_variant=5, block_rows=4), "pairs"), (dict(steps_per_pass=2), "twos"),
+             (dict(), "ones"), (dict(prec="f64"), "ones"), (dict(conv=2), "ones"), (dict(diff=3, steps_per_pass=2), "twos")]
+    for kw, kernel in named:
+        s = Lattice(nx, ny, **kw)
+        C.check(s.lib.lbm_set_launch_fixed(s.h, 1))
+        per = 1 if kernel == "ones" else 2
+        assert s.route(20) == dict(dict.fromkeys(ROUTE_KEYS, 0), **{kernel: 20 // per}), kw
+
+
 def test_route_arguments_are_checked():
     s = Lattice(64, 64)
     v = (ctypes.c_int * 5)()
+    assert s.lib.lbm_set_launch_fixed(s.h, 2) == C.LBM_EINVAL
+    assert s.lib.lbm_set_launch_fixed(None, 1) == C.LBM_EINVAL
     assert s.lib.lbm_step_route(None, 1, 152, v) == C.LBM_EINVAL
     assert s.lib.lbm_step_route(s.h, -1, 152, v) == C.LBM_EINVAL
     assert s.lib.lbm_step_route(s.h, 1, -1, v) == C.LBM_EINVAL
