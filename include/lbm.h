@@ -81,8 +81,12 @@ typedef struct {
                                (F32 and BF16S with periodic or ABB walls). LBM_F32
                                and LBM_F64 with an automatic launch (below) may take
                                more steps per sweep in either case: the populations are the
-                               same bit for bit, and a call's launches stay even or
-                               odd in number as without it                        */
+                               same bit for bit however many steps a call or a sweep
+                               takes, and a call's launches stay even or odd in number
+                               as without it. LBM_F32 with per_cell_K: the same within
+                               each value of steps_per_pass (with 1 always one step
+                               per launch); between the two they differ in the
+                               last bit                                           */
     int per_cell_K;         /* 1: K comes from lbm_set_K_field                    */
     int kernel_variant;     /* 0: automatic (LBM_F32 and LBM_F64 with block_rows 0,
                                Scheme B, conv 0 / 1, diff 0 to 2: the library

@@ -10,21 +10,22 @@
 
 namespace lbm {
 
-// KF: a per-node tensor field, a kernel of its own, since in FP32 it takes another
-// collision and other walls. 2636 x 1533, conv 0, FP32: 5,003 us per pass; with both
+// KF: 0 a constant tensor, 1 a per-node tensor field, 2 a field in FP32 with one step per
+// pass, which takes another collision and other walls; kernels of their own. 2636 x 1533, conv 0, FP32: 5,003 us per pass; with both
 // collisions in one kernel and the walls of both from the table 5,432, with collide()
 // and wall_term() for both 5,067.
-template <int PREC, int CONV, int DIFF, bool KF>
+template <int PREC, int CONV, int DIFF, int KF>
 __global__ void __launch_bounds__(256)
 k_step(const Params<typename Store<PREC>::C> p, const typename Store<PREC>::T *__restrict__ src,
        const float *__restrict__ src_phi, typename Store<PREC>::T *__restrict__ dst, float *__restrict__ dst_phi)
 {
     using S = Store<PREC>;
     using C = typename S::C;
-    // FP32 with a per-node tensor keeps collide() and wall_term(): these are the forward
-    // states of the adjoint, whose gradient in u is a sum of cancelling terms that
-    // magnifies a change of the last bit
-    constexpr int NP = KF && PREC == LBM_F32 ? LBM_BF16S : PREC;
+    // FP32 with a per-node tensor and one step per pass keeps collide() and wall_term():
+    // these are the forward states of the adjoint, whose gradient in u is a sum of
+    // cancelling terms that magnifies a change of the last bit. With two steps per pass the
+    // single steps are the remainder of longer sweeps and take their collision.
+    constexpr int NP = KF == 2 ? LBM_BF16S : PREC;
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
     if (x >= p.nx || y >= p.ny) return;
@@ -69,7 +70,7 @@ k_step(const Params<typename Store<PREC>::C> p, const typename Store<PREC>::T *_
     }
 
     C phi;
-    if constexpr (KF)
+    if constexpr (KF != 0)
         collide_stored<NP, C, CONV, DIFF, true>(
             p, f, __ldg(p.Afield + own), __ldg(p.Afield + P + own), __ldg(p.Afield + 2 * P + own), phi);
     else
@@ -88,8 +89,16 @@ static cudaError_t step_t(const lbm_solver *s, const void *src, const float *src
     const int by = s->d.block_rows > 0 ? s->d.block_rows : 8;
     dim3 block(32, by);
     dim3 grid((s->d.nx + 31) / 32, (s->d.ny + by - 1) / by);
-    if (p.Afield) k_step<PREC, CONV, DIFF, true><<<grid, block, 0, st>>>(p, (const T *)src, src_h, (T *)dst, dst_h);
-    else k_step<PREC, CONV, DIFF, false><<<grid, block, 0, st>>>(p, (const T *)src, src_h, (T *)dst, dst_h);
+    if (!p.Afield) {
+        k_step<PREC, CONV, DIFF, 0><<<grid, block, 0, st>>>(p, (const T *)src, src_h, (T *)dst, dst_h);
+        return cudaGetLastError();
+    }
+    if constexpr (PREC == LBM_F32)
+        if (s->d.steps_per_pass == 1) {
+            k_step<PREC, CONV, DIFF, 2><<<grid, block, 0, st>>>(p, (const T *)src, src_h, (T *)dst, dst_h);
+            return cudaGetLastError();
+        }
+    k_step<PREC, CONV, DIFF, 1><<<grid, block, 0, st>>>(p, (const T *)src, src_h, (T *)dst, dst_h);
     return cudaGetLastError();
 }
 

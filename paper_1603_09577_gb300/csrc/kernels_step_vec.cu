@@ -201,8 +201,9 @@ k_step_v4(const Params<float> p, const typename VecIO<PREC>::T *__restrict__ src
                 const bool ox = p.abb_x && (xs < 0 || xs >= p.nx);
                 const bool oy = p.abb_y && (ys < 0 || ys >= p.ny);
                 if (ox || oy) {
-                    f[c][k] = wall_value<PREC, float, CONV, DIFF>(p, k, ox, oy) -
-                              S::ld(src + opp(k) * P, own, src_h, wgt<float>(opp(k)));
+                    const float even = p.Afield ? wall_value<LBM_BF16S, float, CONV, DIFF>(p, k, ox, oy)
+                                                : wall_value<PREC, float, CONV, DIFF>(p, k, ox, oy);
+                    f[c][k] = even - S::ld(src + opp(k) * P, own, src_h, wgt<float>(opp(k)));
                 }
             }
         }
@@ -226,9 +227,9 @@ k_step_v4(const Params<float> p, const typename VecIO<PREC>::T *__restrict__ src
     }
 
     float phi[4];
-    if (p.Afield) {
+    if (p.Afield) {                      // one step per pass: the collision of kernels_step.cu
 #pragma unroll
-        for (int c = 0; c < 4; ++c) collide_stored<PREC, float, CONV, DIFF, true>(p, f[c], A3[c], A35[c], A5[c], phi[c]);
+        for (int c = 0; c < 4; ++c) collide<float, CONV, DIFF, true>(p, f[c], A3[c], A35[c], A5[c], phi[c]);
     } else {
 #pragma unroll
         for (int c = 0; c < 4; ++c) collide_stored<PREC, float, CONV, DIFF, false>(p, f[c], A3[c], A35[c], A5[c], phi[c]);

@@ -220,8 +220,8 @@ static cudaError_t launch_general(const lbm_solver *s, int src, const double *bv
 // Lattices of Scheme B whose launch is left to the library: FP64 and FP32 with
 // kernel_variant 0 and no block shape, or FP32 with the pair kernels' small tiles
 // (kernel_variant 5, block_rows 4). The kernels of a precision agree bit for bit,
-// whatever the split into sweeps; only with a per-node tensor in FP32 does the
-// one-step kernel differ in the last bit, so that one step per pass stays one there.
+// whatever the split into sweeps; only with a per-node tensor in FP32 and one step per
+// pass do the one-step kernels differ in the last bit, so that they alone run there.
 static bool auto_path(const lbm_solver *s)
 {
     if (s->fixed) return false;
@@ -600,7 +600,9 @@ int lbm_step(lbm_handle h, int nsteps, void *stream)
                              : h->d.kernel_variant == 4 ? launch_step2_tma(h, h->cur, st)
                                                         : launch_step2(h, h->cur, st), 2, "lbm_step (two steps per pass)"))
             return rc;
-    const bool vec = h->d.kernel_variant == 2 || (h->d.kernel_variant == 0 && step_v4_preferred(h));
+    // (in FP32 with a per-node tensor the four-node kernel has the collision of one step per pass only)
+    const bool vec = (h->d.kernel_variant == 2 || (h->d.kernel_variant == 0 && step_v4_preferred(h))) &&
+                     !(h->d.prec == LBM_F32 && h->d.per_cell_K && h->d.steps_per_pass == 2);
     for (int i = 0; i < r.ones; ++i)
         if (int rc = advance(general ? launch_general(h, h->cur, records, nullptr, 0, st)
                              : vec   ? launch_step_v4(h, h->cur, st)
