@@ -91,7 +91,7 @@ static cudaError_t init_t(const lbm_solver *s, const void *phi, int in_prec, cud
     using S = Store<PREC>;
     using T = typename S::T;
     using C = typename S::C;
-    const Params<C> p = make_params<C>(s);
+    const Params<C> &p = make_params<C>(s);
     dim3 block(32, 8), grid((s->d.nx + 31) / 32, (s->d.ny + 7) / 8);
     k_init<PREC, CONV, DIFF><<<grid, block, 0, st>>>(p, phi, in_prec, (T *)s->pop[s->cur], s->phi[s->cur]);
     return cudaGetLastError();
@@ -158,7 +158,7 @@ static cudaError_t get_phi_p(const lbm_solver *s, void *out, int out_prec, cudaS
     using S = Store<PREC>;
     using T = typename S::T;
     using C = typename S::C;
-    const Params<C> p = make_params<C>(s);
+    const Params<C> &p = make_params<C>(s);
     dim3 block(32, 8), grid((s->d.nx + 31) / 32, (s->d.ny + 7) / 8);
     k_get_phi<PREC><<<grid, block, 0, st>>>(p, (const T *)s->pop[s->cur], s->phi[s->cur], out, out_prec);
     return cudaGetLastError();
@@ -318,7 +318,7 @@ static cudaError_t reduce_p(const lbm_solver *s, const double *ref, double *out,
     using S = Store<PREC>;
     using T = typename S::T;
     using C = typename S::C;
-    const Params<C> p = make_params<C>(s);
+    const Params<C> &p = make_params<C>(s);
     k_reduce1<PREC><<<kReduceBlocks, kReduceThreads, 0, st>>>(p, (const T *)s->pop[s->cur], s->phi[s->cur], ref, s->partials);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;

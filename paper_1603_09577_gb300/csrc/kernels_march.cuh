@@ -434,7 +434,7 @@ static cudaError_t march_t(const lbm_solver *s, int src, bool prepare, cudaStrea
     static SmemOptIn once;
     const cudaError_t e = opt_in_smem((const void *)kernel, M::kSmem, once);
     if (e != cudaSuccess || prepare) return e;
-    const Params<float> p = make_params<float>(s);
+    const Params<float> &p = make_params<float>(s);
     MarchArgs a;
     a.k = coll_cast<F2>(p.k);
     a.src = (const float *)s->pop[src];

@@ -85,7 +85,7 @@ static cudaError_t step_t(const lbm_solver *s, const void *src, const float *src
     using S = Store<PREC>;
     using T = typename S::T;
     using C = typename S::C;
-    const Params<C> p = make_params<C>(s);
+    const Params<C> &p = make_params<C>(s);
     const int by = s->d.block_rows > 0 ? s->d.block_rows : 8;
     dim3 block(32, by);
     dim3 grid((s->d.nx + 31) / 32, (s->d.ny + by - 1) / by);

@@ -277,7 +277,7 @@ static cudaError_t step2_ty(const lbm_solver *s, int src, cudaStream_t st)
         const cudaError_t e = opt_in_smem((const void *)k_step2<PREC, CONV, DIFF, TY, KF>, (int)smem, once);
         if (e != cudaSuccess) return e;
     }
-    const Params<float> p = make_params<float>(s);
+    const Params<float> &p = make_params<float>(s);
     dim3 block(32, kT2Threads / 32);
     dim3 grid((s->d.nx + kTX - 1) / kTX, (s->d.ny + TY - 1) / TY);
     k_step2<PREC, CONV, DIFF, TY, KF><<<grid, block, smem, st>>>(p, (const T *)s->pop[src], s->phi[src],

@@ -195,7 +195,7 @@ cudaError_t step2_tma_t(const lbm_solver *s, int src, cudaStream_t st)
     if (e != cudaSuccess) return e;
     CUtensorMap map;
     if (!make_map(&map, s, s->pop[src])) return cudaErrorInvalidValue;
-    const Params<float> p = make_params<float>(s);
+    const Params<float> &p = make_params<float>(s);
     dim3 block(32, kT2Threads / 32);
     dim3 grid((s->d.nx + kTX - 1) / kTX, (s->d.ny + 29) / 30);
     k_step2_tma<CONV, DIFF, KF><<<grid, block, kTmaSmem, st>>>(p, map, (const float *)s->pop[src],

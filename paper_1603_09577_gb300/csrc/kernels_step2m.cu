@@ -225,7 +225,7 @@ template <int PREC, int CONV, int DIFF>
 static cudaError_t step2m_t(const lbm_solver *s, int src, int H, cudaStream_t st)
 {
     using T = typename Store<PREC>::T;
-    const Params<float> p = make_params<float>(s);
+    const Params<float> &p = make_params<float>(s);
     dim3 block(32, kWarpsM);
     const int segs = (s->d.ny + H - 1) / H;
     dim3 grid((s->d.nx + kStripW - 1) / kStripW, (segs + kWarpsM - 1) / kWarpsM);

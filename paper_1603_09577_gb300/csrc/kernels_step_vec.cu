@@ -241,7 +241,7 @@ template <int PREC, int CONV, int DIFF>
 static cudaError_t step_v4_t(const lbm_solver *s, int src, cudaStream_t st)
 {
     using T = typename VecIO<PREC>::T;
-    const Params<float> p = make_params<float>(s);
+    const Params<float> &p = make_params<float>(s);
     const int by = s->d.block_rows > 0 ? s->d.block_rows : 8;
     dim3 block(32, by);
     dim3 grid((s->d.nx + 127) / 128, (s->d.ny + by - 1) / by);

@@ -215,7 +215,7 @@ static cudaError_t tile_t(const lbm_solver *s, int src, int steps, bool prepare,
     static SmemOptIn once;
     const cudaError_t e = opt_in_smem((const void *)k_tile<R, CONV, DIFF, KF>, kTileSmem, once);
     if (e != cudaSuccess || prepare) return e;
-    const Params<R> p = make_params<R>(s);
+    const Params<R> &p = make_params<R>(s);
     TileArgs<R> a;
     a.k = coll_cast<typename TileVec<R>::V>(p.k);
     a.src = (const R *)s->pop[src];

@@ -25,7 +25,7 @@ namespace lbm {
 
 template <int PREC, int CONV, int DIFF, bool WALLS, bool OFF32>
 __global__ void __launch_bounds__(256)
-k_step3(const Params3<typename St3<PREC>::C> p, const Planes3<typename St3<PREC>::T> pl)
+k_step3(const StepParams3<PREC, WALLS> p, const Planes3<typename St3<PREC>::T> pl)
 {
     using S = St3<PREC>;
     using T = typename S::C;
@@ -133,6 +133,10 @@ struct lbm3_solver {
     int cur = 0;
     size_t state_bytes = 0;               // populations, then the BF16S shift plane (contiguous)
     double G[6] = {0, 0, 0, 0, 0, 0};
+    // the kernels' parameters in the compute type of `prec`, made by lbm3_set_coeffs
+    // (made at every launch they took 2 us of host time, as long as the launch itself)
+    lbm::Params3W<float> pf{};
+    lbm::Params3W<double> pd{};
 };
 
 namespace lbm {
@@ -232,9 +236,14 @@ Coll3<double> make_coll3(const lbm3_solver *s)
 }
 
 template <class T>
-Params3<T> params3(const lbm3_solver *s)
+const Params3W<T> &params3(const lbm3_solver *s);
+template <> inline const Params3W<float> &params3<float>(const lbm3_solver *s) { return s->pf; }
+template <> inline const Params3W<double> &params3<double>(const lbm3_solver *s) { return s->pd; }
+
+template <class T>
+Params3W<T> compute_params3(const lbm3_solver *s)
 {
-    Params3<T> p;
+    Params3W<T> p{};
     p.nx = s->d.nx; p.ny = s->d.ny; p.nz = s->d.nz;
     p.pitch = s->pitch; p.plane = s->plane;
     p.se = (T)s->c.se;
@@ -268,6 +277,7 @@ Params3<T> params3(const lbm3_solver *s)
     for (int i = 0; i < 6; ++i) p.phi_wall[i] = (T)s->d.phi_wall[i];
     p.err = s->err;
     p.k = coll3_cast<T>(make_coll3(s));
+    if (!p.any_abb || s->d.prec == LBM_BF16S) return p;        // BF16S forms the wall terms itself
     for (int k = 1; k < 19; ++k)
         for (int set = 1; set < 8; ++set) {
             double tot = 0.0;
@@ -317,7 +327,7 @@ template <int PREC, int CONV, int DIFF>
 cudaError_t launch3_t(const lbm3_solver *s, const void *phi0, int in_prec, cudaStream_t st)
 {
     using T = typename St3<PREC>::T;
-    const auto p = params3<typename St3<PREC>::C>(s);
+    const auto &p = params3<typename St3<PREC>::C>(s);
     if (phi0) {
         // the initial state goes to the current buffer
         Planes3<T> pl = planes3<T>(s);
@@ -370,7 +380,7 @@ cudaError_t sweep3_t(const lbm3_solver *s, bool prepare, cudaStream_t st)
     static SmemOptIn once;
     const cudaError_t e = opt_in_smem((const void *)k_sweep3<CONV, DIFF, SRC, TY, MINB>, S3<TY>::kSmem, once);
     if (e != cudaSuccess || prepare) return e;
-    const Params3<float> p = params3<float>(s);
+    const Params3<float> &p = params3<float>(s);
     Sweep3Args a;
     a.k = coll3_cast<F2>(p.k);
     a.src = (const float *)s->pop[s->cur];
@@ -506,6 +516,8 @@ int lbm3_set_coeffs(lbm3_handle h, const lbm3_coeffs *c)
     // G = A - s_e I
     h->G[0] = A[0] - c->se; h->G[1] = A[1]; h->G[2] = A[2];
     h->G[3] = A[3] - c->se; h->G[4] = A[4]; h->G[5] = A[5] - c->se;
+    if (h->d.prec == LBM_F64) h->pd = compute_params3<double>(h);
+    else h->pf = compute_params3<float>(h);
     h->coeffs_set = 1;
     return LBM_OK;
 }

@@ -5,6 +5,8 @@
 // node with periodic wrap and anti-bounce-back walls.
 #pragma once
 
+#include <type_traits>
+
 #include <cuda_bf16.h>
 
 #include "lbm3.h"
@@ -166,10 +168,19 @@ struct Params3 {
     C phi_wall[6];                   // x-, x+, y-, y+, z-, z+
     int *err;                        // checked builds: index-fault word
     Coll3<C> k;
-    // feq_k + feq_opp(k) at the wall of direction k = 1..18, by the set of axes whose
-    // walls its link crosses (bit a: axis a; the mean value of the walls)
+};
+
+// With walls: feq_k + feq_opp(k) at the wall of direction k = 1..18, by the set of axes
+// whose walls its link crosses (bit a: axis a; the mean value of the walls). Only the
+// kernels that read it take it: up to a kilobyte of kernel arguments per launch (periodic
+// FP64, host time per launch 2.39 us with it, 2.02 before there was a table).
+template <class C>
+struct Params3W : Params3<C> {
     C wt[18][7];
 };
+template <int PREC, bool WALLS>
+using StepParams3 = std::conditional_t<WALLS && PREC != LBM_BF16S, Params3W<typename St3<PREC>::C>,
+                                       Params3<typename St3<PREC>::C>>;
 
 // Coefficients at phi (Eq. 7 families, D = g(phi) I): B, B', the tensor
 // Q = C + c_s^2 g I - c_s^2 phi I of Eq. 3 and trQ/3, and R = r0 + r1 phi.
@@ -324,7 +335,7 @@ __device__ __forceinline__ void collide3(const Params3<C> &p, C f[19], C &phi_ou
 // direction k is the node's own index plus the offsets of its neighbour on
 // each axis, in 32-bit arithmetic (a plane holds fewer than 2^31 elements).
 template <int PREC, int CONV, int DIFF, bool WALLS, bool OFF32>
-__device__ __forceinline__ void pull3_node(const Params3<typename St3<PREC>::C> &p,
+__device__ __forceinline__ void pull3_node(const StepParams3<PREC, WALLS> &p,
                                            const Planes3<typename St3<PREC>::T> &pl, int x, int y, int z,
                                            unsigned own, typename St3<PREC>::C f[19])
 {
@@ -391,7 +402,7 @@ __device__ __forceinline__ void pull3_node(const Params3<typename St3<PREC>::C> 
                 if (p.abb[0] && (xs < 0 || xs >= p.nx)) { tot += xs < 0 ? p.phi_wall[0] : p.phi_wall[1]; ++cnt; }
                 if (p.abb[1] && (ys < 0 || ys >= p.ny)) { tot += ys < 0 ? p.phi_wall[2] : p.phi_wall[3]; ++cnt; }
                 if (p.abb[2] && (zs < 0 || zs >= p.nz)) { tot += zs < 0 ? p.phi_wall[4] : p.phi_wall[5]; ++cnt; }
-                if (PREC != LBM_BF16S) {
+                if constexpr (PREC != LBM_BF16S) {
                     const int set = (p.abb[0] && (xs < 0 || xs >= p.nx) ? 1 : 0) |
                                     (p.abb[1] && (ys < 0 || ys >= p.ny) ? 2 : 0) |
                                     (p.abb[2] && (zs < 0 || zs >= p.nz) ? 4 : 0);

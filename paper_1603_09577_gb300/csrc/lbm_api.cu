@@ -153,9 +153,9 @@ static void wall_table(const lbm_solver *s, C wt[8][3])
 }
 
 template <class C>
-Params<C> make_params(const lbm_solver *s)
+static Params<C> compute_params(const lbm_solver *s)
 {
-    Params<C> p;
+    Params<C> p{};
     const lbm_coeffs &c = s->c;
     p.nx = s->d.nx;
     p.ny = s->d.ny;
@@ -195,12 +195,10 @@ Params<C> make_params(const lbm_solver *s)
     p.bv = nullptr;
     if (p.fisher) p.has_src = 1;
     p.k = coll_cast<C>(make_coll(c, A3, A35, A5));
-    wall_table<C>(s, p.wt);
+    if ((p.abb_x || p.abb_y) && s->d.prec != LBM_BF16S) wall_table<C>(s, p.wt);   // BF16S forms the terms itself
     return p;
 }
 
-template Params<float> make_params<float>(const lbm_solver *);
-template Params<double> make_params<double>(const lbm_solver *);
 
 // the general kernel serves Scheme A, extrapolation walls and the power-law flux
 static bool general_path(const lbm_solver *s)
@@ -481,6 +479,8 @@ int lbm_set_coeffs(lbm_handle h, const lbm_coeffs *c)
         if (!relax_block(c->K, &a, &b, &d)) return fail(LBM_EINVAL, "K is not symmetric positive definite");
     }
     h->c = *c;
+    if (h->d.prec == LBM_F64) h->pd = compute_params<double>(h);
+    else h->pf = compute_params<float>(h);
     h->plan.T = 0;                       // the family decides which kernels serve it
     h->coeffs_set = 1;
     return LBM_OK;

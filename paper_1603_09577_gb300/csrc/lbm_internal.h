@@ -59,6 +59,10 @@ struct lbm_solver {
     int fixed = 0;                  // 1: the kernels that the descriptor names, whatever the size
     int sms = 0;                    // SMs of the device, read at the first step
     lbm::TilePlan plan{0, 0, 0, 0.0};
+    // the kernels' parameters in the compute type of `prec`, made by lbm_set_coeffs (made at
+    // every launch they took 0.1 us of host time of 2.1)
+    lbm::Params<float> pf{};
+    lbm::Params<double> pd{};
     long long t = 0;
     // Dirichlet records of the extrapolated axes (caller-owned device memory)
     const double *dir_vals = nullptr;
@@ -92,7 +96,9 @@ int cuda_check(cudaError_t e, const char *what);
 
 // kernel parameters in the compute type of the solver
 template <class C>
-Params<C> make_params(const lbm_solver *s);
+const Params<C> &make_params(const lbm_solver *s);
+template <> inline const Params<float> &make_params<float>(const lbm_solver *s) { return s->pf; }
+template <> inline const Params<double> &make_params<double>(const lbm_solver *s) { return s->pd; }
 
 // Family key of the step launchers: conv * 3 + diff, or 6 + diff for the linear
 // family without a flux (conv 0 with u = 0), which runs the collision without
