@@ -266,6 +266,14 @@ static cudaError_t launch_march(const lbm_solver *s, int src, bool prepare, cuda
     return launch_march_free(s, src, prepare, st);
 }
 
+static void need_plan(lbm_solver *s, bool general, int sms)
+{
+    if (s->plan.T != 0 && s->plan.general == general && s->plan.sms == sms) return;
+    s->plan = tile_plan(s->d.nx, s->d.ny, s->d.prec == LBM_F64, general, sms);
+    s->plan.general = general;
+    s->plan.sms = sms;
+}
+
 static int device_sms(lbm_solver *s)
 {
     if (s->sms > 0) return LBM_OK;
@@ -292,7 +300,7 @@ static bool tile_general_wanted(lbm_solver *s, int sms)
 {
     if (s->fixed || s->d.kernel_variant != 0 || s->d.block_rows != 0 || s->c.cfree || s->d.prec == LBM_BF16S || s->c.conv > 2) return false;
     if ((long long)s->d.nx * s->d.ny > (s->d.prec == LBM_F64 ? 500000 : 250000)) return false;
-    if (s->plan.T == 0) s->plan = tile_plan(s->d.nx, s->d.ny, s->d.prec == LBM_F64, true, sms);
+    need_plan(s, true, sms);
     return s->plan.us < 1e29 && (s->d.prec == LBM_F64 || s->plan.T >= 2);
 }
 
@@ -339,7 +347,7 @@ static Route plan_route(lbm_solver *h, int nsteps, int sms)
         }
         return r;
     }
-    if (h->plan.T == 0) h->plan = tile_plan(h->d.nx, h->d.ny, h->d.prec == LBM_F64, false, sms);
+    need_plan(h, false, sms);
     if (tile_wanted(h, sms)) {
         r.tiles = tile_launches(h, nsteps);
         return r;
@@ -481,7 +489,6 @@ int lbm_set_coeffs(lbm_handle h, const lbm_coeffs *c)
     h->c = *c;
     if (h->d.prec == LBM_F64) h->pd = compute_params<double>(h);
     else h->pf = compute_params<float>(h);
-    h->plan.T = 0;                       // the family decides which kernels serve it
     h->coeffs_set = 1;
     return LBM_OK;
 }
@@ -632,10 +639,7 @@ int lbm_step_route(lbm_handle h, int nsteps, int sms, int launches[5])
         if (int rc = device_sms(h)) return rc;
         sms = h->sms;
     }
-    const TilePlan kept = h->plan;       // the handle's own plan is for its device's SMs
-    if (sms != h->sms) h->plan.T = 0;
     const Route r = plan_route(h, nsteps, sms);
-    if (sms != h->sms) h->plan = kept;
     const int n[5] = {r.tiles, r.fours, r.pairs, r.twos, r.ones};
     for (int i = 0; i < 5; ++i) launches[i] = n[i];
     return LBM_OK;

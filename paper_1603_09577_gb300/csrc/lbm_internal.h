@@ -32,10 +32,14 @@ int make_layout(const lbm_desc *d, Layout *L);
 namespace lbm {
 
 // Launch of a small lattice: W x H tiles, T steps per launch (kernels_tile.cuh); us:
-// the estimated time of a step. T = 0: not planned yet.
+// the estimated time of a step. T = 0: not planned yet. The search takes 15 to 100 us of
+// host time and depends on the sizes, the precision, the path and the device only, not on
+// the coefficients: a program that changes them as it goes searches once.
 struct TilePlan {
     int W = 0, H = 0, T = 0;
     double us = 0.0;
+    bool general = false;           // for the general path's kernel
+    int sms = 0;                    // for a device of so many SMs
 };
 
 }  // namespace lbm
@@ -58,7 +62,7 @@ struct lbm_solver {
     int cur = 0;
     int fixed = 0;                  // 1: the kernels that the descriptor names, whatever the size
     int sms = 0;                    // SMs of the device, read at the first step
-    lbm::TilePlan plan{0, 0, 0, 0.0};
+    lbm::TilePlan plan;
     // the kernels' parameters in the compute type of `prec`, made by lbm_set_coeffs (made at
     // every launch they took 0.1 us of host time of 2.1)
     lbm::Params<float> pf{};

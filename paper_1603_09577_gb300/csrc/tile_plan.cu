@@ -12,7 +12,8 @@ namespace lbm {
 // T = 4 16.7, T = 8 32; FP64 64^2 T = 3 10.5, 128^2 T = 2 10.4, T = 4 24.9, 200^2 T = 2 18.6.
 TilePlan tile_plan(int nx, int ny, bool f64, bool general, int sms)
 {
-    TilePlan best{nx, ny, 1, 1e30};                  // no tiling fits: never the fastest
+    TilePlan best;
+    best.W = nx; best.H = ny; best.T = 1; best.us = 1e30;          // no tiling fits: never the fastest
     for (int T = 1; T <= kTileMaxT; ++T)
         for (int bx = 1; bx <= nx && bx <= 4 * sms; ++bx) {
             const int W = (nx + bx - 1) / bx;
@@ -33,7 +34,7 @@ TilePlan tile_plan(int nx, int ny, bool f64, bool general, int sms)
                     else t += f64 ? 0.2 + 2.2 * ((warps + 3) / 4) : 0.25 + 0.055 * warps;
                 }
                 const double us = ((f64 ? 3.0 : 4.5) + n_waves * t) / T;
-                if (us < best.us) best = TilePlan{W, H, T, us};
+                if (us < best.us) { best.W = W; best.H = H; best.T = T; best.us = us; }
             }
         }
     return best;

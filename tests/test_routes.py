@@ -3,6 +3,7 @@ lbm3_step_route): every route adds up to the steps asked for, keeps the number o
 launches odd or even as steps_per_pass has it (captured calls then end on the buffer
 they started from), and is what the benchmark's records name."""
 import ctypes
+import time
 
 import pytest
 
@@ -81,6 +82,30 @@ def test_routes_add_up_and_keep_the_parity(kind, walls):
                     assert fixed == n, (nx, ny, n, r)
                 wanted = n // 2 + n % 2 if spp == 2 else n
                 assert sum(r.values()) % 2 == wanted % 2, (nx, ny, n, r)
+
+
+@pytest.mark.parametrize("kw", [dict(nx=20000, ny=12), dict(nx=20000, ny=12, prec="f64"),
+                                dict(nx=20000, ny=12, conv=2)], ids=["f32", "f64", "general"])
+def test_changed_coefficients_do_not_search_the_tiling_again(kw):
+    def least(fn):
+        best = float("inf")
+        for _ in range(50):
+            t = time.perf_counter()
+            fn()
+            best = min(best, time.perf_counter() - t)
+        return best
+
+    s = Lattice(**kw)
+    conv = kw.get("conv", 0)
+    s.route(10)
+
+    def change():
+        s.set_coeffs(conv=conv, u=(0.01, 0.02))
+        s.route(10)
+
+    search = least(lambda: Lattice(**kw).route(10)) - least(lambda: Lattice(**kw))
+    assert search > 10e-6                                     # what a repeated search would cost
+    assert least(change) - least(lambda: s.set_coeffs(conv=conv, u=(0.01, 0.02))) < 0.2 * search
 
 
 def test_the_benchmark_names_the_kernel_that_runs():
