@@ -11,11 +11,18 @@
 namespace lbm {
 
 // KF: 0 a constant tensor, 1 a per-node tensor field, 2 a field in FP32 with one step per
-// pass, which takes another collision and other walls; kernels of their own. 2636 x 1533, conv 0, FP32: 5,003 us per pass; with both
-// collisions in one kernel and the walls of both from the table 5,432, with collide()
-// and wall_term() for both 5,067.
+// pass, which takes another collision and other walls; kernels of their own. 2636 x 1533,
+// conv 0, FP32, 100 steps with a field: 5,003 us per pass; with both collisions in one kernel
+// and the walls of both from the table 5,432, with collide() and wall_term() for both 5,067.
+//
+// FP32 families whose collision fits into 32 registers (all but the quadratic flux) are held
+// to them: eight blocks per SM, the loads in flight that HBM's rate takes. Left alone the
+// compiler gave relax() 38 to 40 registers and six blocks: 4096^2 185.5 us against 177.2,
+// 1024^2 11.2 against 10.3 (the kernel on collide(): 178.0 and 12.3).
+template <int PREC, int CONV> constexpr int kStepBlocks = PREC == LBM_F32 && CONV != 1 ? 8 : 0;
+
 template <int PREC, int CONV, int DIFF, int KF>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, kStepBlocks<PREC, CONV>)
 k_step(const Params<typename Store<PREC>::C> p, const typename Store<PREC>::T *__restrict__ src,
        const float *__restrict__ src_phi, typename Store<PREC>::T *__restrict__ dst, float *__restrict__ dst_phi)
 {
