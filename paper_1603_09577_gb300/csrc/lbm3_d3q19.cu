@@ -23,8 +23,13 @@
 
 namespace lbm {
 
-template <int PREC, int CONV, int DIFF, bool WALLS, bool OFF32>
-__global__ void __launch_bounds__(256)
+// SRC: there is a source (BF16S decides at run time). FP64 is bound by its pipe and held to
+// 64 registers, four blocks per SM; FP32 to 40, six blocks. With both forms of relax3() in
+// one kernel and 80 registers in FP64 (three blocks), against now (us per step): 256 x 256 x
+// 128 FP64 cubic diffusion with a source 2044 -> 1968, without 1937 -> 1905; 59 x 74 x 27
+// with a source 42.7 -> 41.0; 64^3 FP32 8.2 -> 6.5.
+template <int PREC, int CONV, int DIFF, bool WALLS, bool OFF32, bool SRC>
+__global__ void __launch_bounds__(256, PREC == LBM_F64 ? 4 : (PREC == LBM_F32 ? 6 : 0))
 k_step3(const StepParams3<PREC, WALLS> p, const Planes3<typename St3<PREC>::T> pl)
 {
     using S = St3<PREC>;
@@ -38,8 +43,7 @@ k_step3(const StepParams3<PREC, WALLS> p, const Planes3<typename St3<PREC>::T> p
     pull3_node<PREC, CONV, DIFF, WALLS, OFF32>(p, pl, x, y, z, own, f);
     T phi = T(0), mass = T(0);
     if constexpr (PREC != LBM_BF16S) {
-        if (p.has_src) relax3<T, CONV, DIFF, true>(p.k, f);
-        else relax3<T, CONV, DIFF, false>(p.k, f);
+        relax3<T, CONV, DIFF, SRC>(p.k, f);
     } else {
         collide3<CONV, DIFF, T>(p, f, phi, mass);
     }
@@ -205,7 +209,7 @@ bool relax_block3(const double K[6], double A[6])
 
 Coll3<double> make_coll3(const lbm3_solver *s)
 {
-    Coll3<double> k;
+    Coll3<double> k{};
     const double se = s->c.se, *u = s->c.u, u2_3 = (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]) / 3.0;
     const bool quad = s->c.conv == 1;                 // B = a phi^2/2, C = a a phi^3/3
     const double half = quad ? 0.5 : 1.0, third = quad ? 1.0 / 3.0 : 1.0;
@@ -232,6 +236,15 @@ Coll3<double> make_coll3(const lbm3_solver *s)
     k.inv_den = 1.0 / (1.0 - 0.5 * s->c.r1);
     k.phi0 = 0.5 * s->c.r0 * k.inv_den;
     k.r0 = s->c.r0; k.r1 = s->c.r1;
+    if (!quad) {                                      // R = r0 + r1 phi: the source joins the other terms in phi
+        for (int a = 0; a < 3; ++a) {
+            k.nb[a] += k.ph[a] * k.r1;
+            k.pc[a] = k.ph[a] * k.r0;
+        }
+        k.tb += k.hse * k.r1;
+        k.xs += k.hse * k.r1;
+        k.hr0 = k.hse * k.r0;
+    }
     return k;
 }
 
@@ -337,10 +350,15 @@ cudaError_t launch3_t(const lbm3_solver *s, const void *phi0, int in_prec, cudaS
     } else {
         const bool off32 = 19 * s->plane < (1LL << 32);
         const Planes3<T> pl = planes3<T>(s);
-        if (p.any_abb && off32) k_step3<PREC, CONV, DIFF, true, true><<<grid3(s), block3(s), 0, st>>>(p, pl);
-        else if (p.any_abb) k_step3<PREC, CONV, DIFF, true, false><<<grid3(s), block3(s), 0, st>>>(p, pl);
-        else if (off32) k_step3<PREC, CONV, DIFF, false, true><<<grid3(s), block3(s), 0, st>>>(p, pl);
-        else k_step3<PREC, CONV, DIFF, false, false><<<grid3(s), block3(s), 0, st>>>(p, pl);
+        auto launch = [&](auto walls, auto o32) {
+            constexpr bool W = decltype(walls)::value, O = decltype(o32)::value;
+            if (PREC != LBM_BF16S && p.has_src) k_step3<PREC, CONV, DIFF, W, O, PREC != LBM_BF16S><<<grid3(s), block3(s), 0, st>>>(p, pl);
+            else k_step3<PREC, CONV, DIFF, W, O, false><<<grid3(s), block3(s), 0, st>>>(p, pl);
+        };
+        if (p.any_abb && off32) launch(std::true_type(), std::true_type());
+        else if (p.any_abb) launch(std::true_type(), std::false_type());
+        else if (off32) launch(std::false_type(), std::true_type());
+        else launch(std::false_type(), std::false_type());
     }
     return cudaGetLastError();
 }

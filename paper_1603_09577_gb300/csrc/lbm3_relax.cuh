@@ -31,16 +31,23 @@ __device__ __forceinline__ void relax3(const Coll3<C> &k, C f[19])
     if constexpr (CONV == 1 || DIFF != 0) phi2 = vmul(phi, phi);
     if constexpr (CONV == 1 || DIFF == 2) phi3 = vmul(phi2, phi);
     const C beta = CONV == 1 ? phi2 : phi, cphi = CONV == 1 ? phi3 : phi;
-    C R, S;
     C vx = vmad(k.nb[0], beta, jx), vy = vmad(k.nb[1], beta, jy), vz = vmad(k.nb[2], beta, jz);
-    C t = vmul(k.tb, beta);
-    C X = vmul(k.xs, phi);
+    C t, X;
+    if constexpr (SRC && CONV == 0) {
+        vx = vadd(vx, k.pc[0]);
+        vy = vadd(vy, k.pc[1]);
+        vz = vadd(vz, k.pc[2]);
+        t = vmad(k.tb, phi, k.hr0);
+        X = vmad(k.xs, phi, k.hr0);
+    } else {
+        t = vmul(k.tb, beta);
+        X = vmul(k.xs, phi);
+    }
     if constexpr (CONV == 1) X = vmad(k.xc, phi3, X);
     if constexpr (DIFF == 1) X = vmad(k.xi, phi2, X);
     if constexpr (DIFF == 2) X = vmad(k.xi, phi3, X);
-    if constexpr (SRC) {
-        R = vmad(k.r1, phi, k.r0);
-        S = CONV == 1 ? vmul(R, phi) : R;
+    if constexpr (SRC && CONV == 1) {
+        const C R = vmad(k.r1, phi, k.r0), S = vmul(R, phi);
         vx = vmad(k.ph[0], S, vx);
         vy = vmad(k.ph[1], S, vy);
         vz = vmad(k.ph[2], S, vz);
