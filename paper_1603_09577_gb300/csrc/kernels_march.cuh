@@ -52,7 +52,7 @@ struct MarchArgs {
 
 // The one shape in use: four steps per sweep, strips of 128 columns, two warps per
 // level, two staged rows; 64 registers and 55 KB of shared memory, four blocks per SM.
-constexpr int kMarchT = 4, kMarchKW = 2, kMarchP = 1, kMarchStage = 2, kMarchBlocks = 4;
+constexpr int kMarchT = 4, kMarchKW = 2, kMarchP = 1, kMarchStage = 2;
 
 template <int T, int KW, int P, int STAGE> struct March {
     static constexpr int kThreads = 32 * KW * T;
@@ -423,9 +423,6 @@ k_march(const __grid_constant__ MarchArgs a)
     else march_strip<CONV, DIFF, SRC, KF, T, KW, P, ST, false>(a, a.k, sm_m, X0, Y0, Y1, false, false);
 }
 
-// Blocks: one wave of four per SM, or up to three where the chunks stay 48 rows or
-// more (a chunk takes 9 iterations beyond its rows). 4096^2: 1824 blocks 218.5k MLUPS,
-// 608 204.4k, 4000 211.1k; 1024^2 (chunks of 15 rows): 608 blocks 154k, 304 112.7k.
 template <int CONV, int DIFF, int SRC, bool KF>
 static cudaError_t march_t(const lbm_solver *s, int src, bool prepare, cudaStream_t st)
 {
@@ -450,13 +447,11 @@ static cudaError_t march_t(const lbm_solver *s, int src, bool prepare, cudaStrea
         for (int z = 0; z < 3; ++z) a.wt[k][z] = p.wt[k][z];
     a.has_src = p.has_src;
     a.err = p.err;
-    const int wave = s->sms * kMarchBlocks;
-    a.strips = (p.nx + M::kOut - 1) / M::kOut;
-    long long waves = (long long)a.strips * p.ny / (48LL * wave);
-    waves = waves < 1 ? 1 : (waves > 3 ? 3 : waves);
-    const int chunks = (int)(waves * wave / a.strips) > 1 ? (int)(waves * wave / a.strips) : 1;
-    a.H = (p.ny + chunks - 1) / chunks;
-    a.chunks = (p.ny + a.H - 1) / a.H;
+    static_assert(M::kOut == kMarchOut, "strips of the launch's grid");
+    const MarchGrid g = march_grid(p.nx, p.ny, s->sms);
+    a.strips = g.strips;
+    a.chunks = g.chunks;
+    a.H = g.H;
     kernel<<<a.strips * a.chunks, M::kThreads, M::kSmem, st>>>(a);
     return cudaGetLastError();
 }

@@ -19,10 +19,9 @@ namespace lbm {
 // to them: eight blocks per SM, the loads in flight that HBM's rate takes. Left alone the
 // compiler gave relax() 38 to 40 registers and six blocks: 4096^2 185.5 us against 177.2,
 // 1024^2 11.2 against 10.3 (the kernel on collide(): 178.0 and 12.3).
-template <int PREC, int CONV> constexpr int kStepBlocks = PREC == LBM_F32 && CONV != 1 ? 8 : 0;
-
-template <int PREC, int CONV, int DIFF, int KF>
-__global__ void __launch_bounds__(256, kStepBlocks<PREC, CONV>)
+// Rows of a sector or two are the exception (2 x 300000 periodic 92 us, with eight blocks 112).
+template <int PREC, int CONV, int DIFF, int KF, int BLOCKS = 0>
+__global__ void __launch_bounds__(256, BLOCKS)
 k_step(const Params<typename Store<PREC>::C> p, const typename Store<PREC>::T *__restrict__ src,
        const float *__restrict__ src_phi, typename Store<PREC>::T *__restrict__ dst, float *__restrict__ dst_phi)
 {
@@ -96,16 +95,21 @@ static cudaError_t step_t(const lbm_solver *s, const void *src, const float *src
     const int by = s->d.block_rows > 0 ? s->d.block_rows : 8;
     dim3 block(32, by);
     dim3 grid((s->d.nx + 31) / 32, (s->d.ny + by - 1) / by);
+    if constexpr (PREC == LBM_F32 && CONV != 1)
+        if (!p.Afield && s->d.nx > 16) {
+            k_step<PREC, CONV, DIFF, 0, 8><<<grid, block, 0, st>>>(p, (const T *)src, src_h, (T *)dst, dst_h);
+            return cudaGetLastError();
+        }
     if (!p.Afield) {
         k_step<PREC, CONV, DIFF, 0><<<grid, block, 0, st>>>(p, (const T *)src, src_h, (T *)dst, dst_h);
         return cudaGetLastError();
     }
     if constexpr (PREC == LBM_F32)
         if (s->d.steps_per_pass == 1) {
-            k_step<PREC, CONV, DIFF, 2><<<grid, block, 0, st>>>(p, (const T *)src, src_h, (T *)dst, dst_h);
+            k_step<PREC, CONV, DIFF, 2, CONV == 1 ? 0 : 8><<<grid, block, 0, st>>>(p, (const T *)src, src_h, (T *)dst, dst_h);
             return cudaGetLastError();
         }
-    k_step<PREC, CONV, DIFF, 1><<<grid, block, 0, st>>>(p, (const T *)src, src_h, (T *)dst, dst_h);
+    k_step<PREC, CONV, DIFF, 1, PREC == LBM_F32 && CONV != 1 ? 8 : 0><<<grid, block, 0, st>>>(p, (const T *)src, src_h, (T *)dst, dst_h);
     return cudaGetLastError();
 }
 

@@ -285,18 +285,17 @@ static cudaError_t step2_ty(const lbm_solver *s, int src, cudaStream_t st)
     return cudaGetLastError();
 }
 
-// tile height from the descriptor: block_rows 4 selects 30 x 30 tiles, anything
-// else 30 x 62
+// tile height: rows 4 selects 30 x 30 tiles, anything else 30 x 62
 template <int PREC, int CONV, int DIFF>
-static cudaError_t step2_t(const lbm_solver *s, int src, cudaStream_t st)
+static cudaError_t step2_t(const lbm_solver *s, int src, int rows, cudaStream_t st)
 {
     // per-node tensor field or not: a compile-time choice, so the constant-K
     // kernel carries no field loads or their registers
     if (s->d.per_cell_K) {
-        if (s->d.block_rows == 4) return step2_ty<PREC, CONV, DIFF, 30, true>(s, src, st);
+        if (rows == 4) return step2_ty<PREC, CONV, DIFF, 30, true>(s, src, st);
         return step2_ty<PREC, CONV, DIFF, 62, true>(s, src, st);
     }
-    if (s->d.block_rows == 4) return step2_ty<PREC, CONV, DIFF, 30, false>(s, src, st);
+    if (rows == 4) return step2_ty<PREC, CONV, DIFF, 30, false>(s, src, st);
     return step2_ty<PREC, CONV, DIFF, 62, false>(s, src, st);
 }
 

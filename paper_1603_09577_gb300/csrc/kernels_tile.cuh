@@ -23,8 +23,6 @@
 
 namespace lbm {
 
-constexpr int kTileMaxT = 8;
-
 template <class R> struct TileVec;                   // arithmetic type and nodes per item
 template <> struct TileVec<float> { using V = F2; static constexpr int N = 2, kThreads = 768; };
 template <> struct TileVec<double> { using V = double; static constexpr int N = 1, kThreads = 512; };

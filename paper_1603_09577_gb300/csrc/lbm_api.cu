@@ -6,7 +6,6 @@
 #include <stdio.h>
 #include <string.h>
 
-#include <algorithm>
 #include <new>
 #include <string>
 
@@ -200,32 +199,12 @@ static Params<C> compute_params(const lbm_solver *s)
 }
 
 
-// the general kernel serves Scheme A, extrapolation walls and the power-law flux
-static bool general_path(const lbm_solver *s)
-{
-    return s->d.scheme == LBM_SCHEME_A || s->d.bc_x == LBM_NEE || s->d.bc_y == LBM_NEE || s->c.conv >= 2 ||
-           s->c.diff == 3;
-}
-
 static cudaError_t launch_general(const lbm_solver *s, int src, const double *bv, const void *phi0, int in_prec,
                                   cudaStream_t st)
 {
     if (s->d.prec == LBM_F64) return launch_general_f64(s, src, bv, phi0, in_prec, st);
     if (s->d.prec == LBM_F32) return launch_general_f32(s, src, bv, phi0, in_prec, st);
     return cudaErrorInvalidValue;
-}
-
-// Lattices of Scheme B whose launch is left to the library: FP64 and FP32 with
-// kernel_variant 0 and no block shape, or FP32 with the pair kernels' small tiles
-// (kernel_variant 5, block_rows 4). The kernels of a precision agree bit for bit,
-// whatever the split into sweeps; only with a per-node tensor in FP32 and one step per
-// pass do the one-step kernels differ in the last bit, so that they alone run there.
-static bool auto_path(const lbm_solver *s)
-{
-    if (s->fixed) return false;
-    if (s->d.prec == LBM_F64) return s->d.kernel_variant == 0 && s->d.block_rows == 0;
-    return s->d.prec == LBM_F32 && !(s->d.per_cell_K && s->d.steps_per_pass == 1) &&
-           ((s->d.kernel_variant == 0 && s->d.block_rows == 0) || (s->d.kernel_variant == 5 && s->d.block_rows == 4));
 }
 
 static cudaError_t launch_tile(const lbm_solver *s, int src, int steps, bool prepare, cudaStream_t st)
@@ -237,41 +216,11 @@ static cudaError_t launch_tile(const lbm_solver *s, int src, int steps, bool pre
                            : launch_tile_f32_const(s, src, steps, prepare, st);
 }
 
-// Whether the tiles of s->plan are estimated faster per step than the large
-// lattices' kernels (microseconds). FP32, the marching kernel and the pair tiles:
-// 4.14 at 400^2 (tiles 2.18), 4.17 at 600^2 (4.00), 5.74 at 803 x 797 (7.00). FP64, the
-// one-step kernel, whose blocks of 256 nodes take two turns of an SM's FP64 pipe
-// each: 8.28 at 128^2 (tiles 5.21), 14.4 at 200^2 (9.31), 19.0 at 301^2 (16.9).
-static bool tile_wanted(const lbm_solver *s, int sms)
-{
-    const double n = (double)s->d.nx * s->d.ny;
-    if (s->d.prec == LBM_F64) {
-        const long long blocks = (long long)((s->d.nx + 31) / 32) * ((s->d.ny + 7) / 8);
-        return s->plan.us < 3.2 + 5.2 * (double)((blocks + sms - 1) / sms);
-    }
-    return s->plan.us < std::max(4.1, 2.5 + n / 210e3);
-}
-
-// Whether sweeps of four steps by the marching kernel serve this lattice. They need
-// strips and chunks for the whole chip: from about 2^18 nodes on.
-static bool march_wanted(const lbm_solver *s)
-{
-    return s->d.nx >= 128 && s->d.ny >= 64 && (long long)s->d.nx * s->d.ny >= (1LL << 18) && s->L.plane < (1LL << 31);
-}
-
 static cudaError_t launch_march(const lbm_solver *s, int src, bool prepare, cudaStream_t st)
 {
     if (s->d.per_cell_K) return launch_march_kfield(s, src, prepare, st);
     if (s->c.r0 != 0.0 || s->c.r1 != 0.0) return launch_march_src(s, src, prepare, st);
     return launch_march_free(s, src, prepare, st);
-}
-
-static void need_plan(lbm_solver *s, bool general, int sms)
-{
-    if (s->plan.T != 0 && s->plan.general == general && s->plan.sms == sms) return;
-    s->plan = tile_plan(s->d.nx, s->d.ny, s->d.prec == LBM_F64, general, sms);
-    s->plan.general = general;
-    s->plan.sms = sms;
 }
 
 static int device_sms(lbm_solver *s)
@@ -280,28 +229,6 @@ static int device_sms(lbm_solver *s)
     int dev = 0;
     if (int rc = cuda_check(cudaGetDevice(&dev), "cudaGetDevice")) return rc;
     return cuda_check(cudaDeviceGetAttribute(&s->sms, cudaDevAttrMultiProcessorCount, dev), "SM count");
-}
-
-// As few launches of the plan's tiles as hold nsteps, even or odd in number as with
-// steps_per_pass steps each (a captured call then ends on the buffer it started from)
-static int tile_launches(const lbm_solver *s, int nsteps)
-{
-    const int wanted = s->d.steps_per_pass == 2 ? nsteps / 2 + nsteps % 2 : nsteps;
-    const int launches = (nsteps + s->plan.T - 1) / s->plan.T;
-    return ((launches ^ wanted) & 1) && launches < nsteps ? launches + 1 : launches;
-}
-
-// The general path's small lattices (the C-free variant runs one step per launch).
-// Measured on the Burgers-Fisher problem, us per step, other kernel -> tiles: FP32 one
-// step per pass 60^2 4.4 -> 2.0, 301^2 6.4 -> 4.1, 500^2 8.5 -> 7.0, 700^2 10.6 -> 12.7; two
-// 6.4 -> 1.9, 6.4 -> 4.1, 7.7 -> 7.0, 9.8 -> 12.7; FP64 60^2 24.9 -> 11.1, 200^2 45.4 -> 28.1,
-// 500^2 103 -> 97, 700^2 174 -> 165 (there with one step per launch: smaller blocks).
-static bool tile_general_wanted(lbm_solver *s, int sms)
-{
-    if (s->fixed || s->d.kernel_variant != 0 || s->d.block_rows != 0 || s->c.cfree || s->d.prec == LBM_BF16S || s->c.conv > 2) return false;
-    if ((long long)s->d.nx * s->d.ny > (s->d.prec == LBM_F64 ? 500000 : 250000)) return false;
-    need_plan(s, true, sms);
-    return s->plan.us < 1e29 && (s->d.prec == LBM_F64 || s->plan.T >= 2);
 }
 
 static cudaError_t launch_tile_general(const lbm_solver *s, int src, const double *records, int steps, bool prepare,
@@ -313,58 +240,6 @@ static cudaError_t launch_tile_general(const lbm_solver *s, int src, const doubl
                  : launch_tile_general_f64_b(s, src, records, steps, prepare, st);
     return a ? launch_tile_general_f32_a(s, src, records, steps, prepare, st)
              : launch_tile_general_f32_b(s, src, records, steps, prepare, st);
-}
-
-// The launches of a call, in the order they run
-struct Route {
-    int tiles = 0;      // small lattices' tiles, which share their steps as evenly as they can
-    int fours = 0;      // sweeps of four steps (the marching kernel)
-    int pairs = 0;      // sweeps of two steps over pair tiles
-    int twos = 0;       // sweeps of two steps by another kernel (the one that the descriptor names)
-    int ones = 0;       // single steps
-};
-
-// The route of nsteps steps on a device of `sms` SMs. On the path left to the library
-// the number of launches stays odd or even as it is with steps_per_pass steps each (n,
-// or n/2 + n%2), so that a captured call that ended on the buffer it started from
-// still does: with m pairs of steps, sweeps of four are even in number (two steps per
-// pass) or as m (one).
-static Route plan_route(lbm_solver *h, int nsteps, int sms)
-{
-    Route r;
-    if (general_path(h)) {
-        if (tile_general_wanted(h, sms)) r.tiles = tile_launches(h, nsteps);
-        else if (h->d.steps_per_pass == 2) { r.twos = nsteps / 2; r.ones = nsteps % 2; }
-        else r.ones = nsteps;
-        return r;
-    }
-    if (!auto_path(h)) {
-        if (h->d.steps_per_pass == 2) {
-            (h->d.kernel_variant == 5 ? r.pairs : r.twos) = nsteps / 2;
-            r.ones = nsteps % 2;
-        } else {
-            r.ones = nsteps;
-        }
-        return r;
-    }
-    need_plan(h, false, sms);
-    if (tile_wanted(h, sms)) {
-        r.tiles = tile_launches(h, nsteps);
-        return r;
-    }
-    const int m = h->d.prec == LBM_F64 ? 0 : nsteps / 2;
-    if (h->d.prec == LBM_F32 && march_wanted(h)) {
-        r.fours = m / 2;
-        if ((r.fours & 1) != (h->d.steps_per_pass == 2 ? 0 : (m & 1))) --r.fours;
-        if (r.fours < 0) r.fours = 0;
-    }
-    r.pairs = m - 2 * r.fours;
-    r.ones = nsteps - 2 * m;
-    if (h->d.steps_per_pass == 1 && ((r.fours + r.pairs) & 1)) {     // no sweeps of four to make the count even
-        --r.pairs;
-        r.ones += 2;
-    }
-    return r;
 }
 
 static int check_handle(lbm_handle h)
@@ -590,7 +465,7 @@ int lbm_step(lbm_handle h, int nsteps, void *stream)
     };
     h->dir_off = 0;
     for (int left = r.tiles; left > 0; --left) {
-        const int steps = (nsteps - done + left - 1) / left;
+        const int steps = (nsteps - r.ones - done + left - 1) / left;      // with tiles, the rest are single steps
         if (int rc = advance(general ? launch_tile_general(h, h->cur, records, steps, false, st)
                                      : launch_tile(h, h->cur, steps, false, st), steps, "lbm_step (small lattice)"))
             return rc;
@@ -605,7 +480,7 @@ int lbm_step(lbm_handle h, int nsteps, void *stream)
         if (int rc = advance(general                    ? launch_step2_general(h, h->cur, records, st)
                              : h->d.kernel_variant == 3 ? launch_step2m(h, h->cur, st)
                              : h->d.kernel_variant == 4 ? launch_step2_tma(h, h->cur, st)
-                                                        : launch_step2(h, h->cur, st), 2, "lbm_step (two steps per pass)"))
+                                                        : launch_step2(h, h->cur, auto_path(h) ? 4 : h->d.block_rows, st), 2, "lbm_step (two steps per pass)"))
             return rc;
     // (in FP32 with a per-node tensor the four-node kernel has the collision of one step per pass only)
     const bool vec = (h->d.kernel_variant == 2 || (h->d.kernel_variant == 0 && step_v4_preferred(h))) &&

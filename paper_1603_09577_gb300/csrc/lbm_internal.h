@@ -31,15 +31,31 @@ int make_layout(const lbm_desc *d, Layout *L);
 
 namespace lbm {
 
-// Launch of a small lattice: W x H tiles, T steps per launch (kernels_tile.cuh); us:
-// the estimated time of a step. T = 0: not planned yet. The search takes 15 to 100 us of
-// host time and depends on the sizes, the precision, the path and the device only, not on
-// the coefficients: a program that changes them as it goes searches once.
+constexpr int kTileMaxT = 8;        // most steps of a launch over a small lattice's tiles
+
+// The launches that a lattice can take and their estimated times (route.cu). The tiling
+// of the small lattices' kernels: W x H tiles, at most T steps per launch; us: the
+// estimated time of a step (1e30: no tiling fits). The search takes 15 to 100 us of host
+// time and depends on the sizes, the walls, the precision, the path and the device only, not on
+// the coefficients: a program that changes them as it goes searches once. T = 0: not planned yet.
 struct TilePlan {
     int W = 0, H = 0, T = 0;
     double us = 0.0;
     bool general = false;           // for the general path's kernel
     int sms = 0;                    // for a device of so many SMs
+    double launch[kTileMaxT + 1] = {};              // us of a launch of so many steps over the tiles
+    double one = 0.0, two = 0.0, four = 0.0;        // FP32, Scheme B: us of the other kernels' launches
+    bool nodes = false;             // two steps: 30 x 30 node tiles, not 62 x 14 pair tiles
+};
+
+// The launches of a call, in the order they run
+struct Route {
+    int tiles = 0;      // small lattices' tiles, which share their steps as evenly as they can
+    int fours = 0;      // sweeps of four steps (the marching kernel)
+    int pairs = 0;      // sweeps of two steps over pair tiles
+    int twos = 0;       // sweeps of two steps by another kernel: the one that the descriptor
+                        // names, or on the path left to the library 30 x 30 node tiles
+    int ones = 0;       // single steps
 };
 
 }  // namespace lbm
@@ -164,7 +180,8 @@ inline Coll<double> make_coll(const lbm_coeffs &c, double A3, double A35, double
 
 cudaError_t launch_init(const lbm_solver *s, const void *phi, int in_prec, cudaStream_t st);
 cudaError_t launch_step(const lbm_solver *s, int src, cudaStream_t st);
-cudaError_t launch_step2(const lbm_solver *s, int src, cudaStream_t st);
+// node tiles of two steps; rows: lbm_desc.block_rows (4: 30 x 30, else 30 x 62)
+cudaError_t launch_step2(const lbm_solver *s, int src, int rows, cudaStream_t st);
 cudaError_t launch_step2m(const lbm_solver *s, int src, cudaStream_t st);
 cudaError_t launch_step2_tma(const lbm_solver *s, int src, cudaStream_t st);
 // two steps per pass, two x-adjacent nodes per thread (kernel_variant 5)
@@ -188,6 +205,15 @@ cudaError_t launch_march_free(const lbm_solver *s, int src, bool prepare, cudaSt
 cudaError_t launch_march_kfield(const lbm_solver *s, int src, bool prepare, cudaStream_t st);
 // `steps` steps in one launch over the tiles of s->plan (kernels_tile.cuh)
 TilePlan tile_plan(int nx, int ny, bool f64, bool general, int sms);
+double tile_launch_us(int nx, int ny, int W, int H, int steps, bool f64, bool general, int sms);
+// the route of nsteps steps on a device of `sms` SMs, and whether the launch is left to the library
+bool general_path(const lbm_solver *s);
+bool auto_path(const lbm_solver *s);
+Route plan_route(lbm_solver *s, int nsteps, int sms);
+// strips and chunks of the marching kernel's launch: blocks of H rows, four per SM
+constexpr int kMarchBlocks = 4, kMarchOut = 120;
+struct MarchGrid { int strips, chunks, H; };
+MarchGrid march_grid(int nx, int ny, int sms);
 #define LBM_DECLARE_TILE_GENERAL(NAME) \
     cudaError_t NAME(const lbm_solver *s, int src, const double *records, int steps, bool prepare, cudaStream_t st)
 LBM_DECLARE_TILE_GENERAL(launch_tile_general_f32_a);
