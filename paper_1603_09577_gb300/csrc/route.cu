@@ -124,6 +124,12 @@ static void need_plan(lbm_solver *s, bool general, int sms)
         for (int n = 1; n <= s->plan.T; ++n)
             s->plan.launch[n] = tile_launch_us(s->d.nx, s->d.ny, s->plan.W, s->plan.H, n, f64, general, sms);
     if (!f64 && !general) estimate(s, sms, &s->plan);
+    if (!f64 && general) {               // one step: 32 x 4 tiles; several: 30 % more at walls
+        const double blocks = (double)((s->d.nx + 31) / 32) * ((s->d.ny + 3) / 4);
+        const bool walls = s->d.bc_x != LBM_PERIODIC || s->d.bc_y != LBM_PERIODIC;
+        for (double &us : s->plan.launch) us *= walls ? 1.3 : 1.0;
+        s->plan.launch[1] = std::max(4.1, (walls ? 4.6 : 3.4) + 1.6e-3 * blocks);
+    }
 }
 
 // launches of a call, modulo 2: as with steps_per_pass steps each (n, or n/2 + n%2), so that
@@ -151,24 +157,38 @@ static int tile_launches(const lbm_solver *s, int nsteps, int parity, int least,
     return best;
 }
 
-// As few launches of the plan's tiles as hold nsteps
-static int fewest_tile_launches(const lbm_solver *s, int nsteps)
-{
-    const int launches = (nsteps + s->plan.T - 1) / s->plan.T;
-    return ((launches ^ launch_parity(s, nsteps)) & 1) && launches < nsteps ? launches + 1 : launches;
-}
-
-// The general path's small lattices (the C-free variant runs one step per launch).
-// Measured on the Burgers-Fisher problem, us per step, other kernel -> tiles: FP32 one
-// step per pass 60^2 4.4 -> 2.0, 301^2 6.4 -> 4.1, 500^2 8.5 -> 7.0, 700^2 10.6 -> 12.7; two
-// 6.4 -> 1.9, 6.4 -> 4.1, 7.7 -> 7.0, 9.8 -> 12.7; FP64 60^2 24.9 -> 11.1, 200^2 45.4 -> 28.1,
-// 500^2 103 -> 97, 700^2 174 -> 165 (there with one step per launch: smaller blocks).
+// The general path's small lattices (the C-free variant runs one step per launch). All
+// calls of a lattice take the same kernel, tiles or not: its bits differ from the other
+// general kernels' in the last place. Measured on a power-law flux, us per step in calls of
+// 20 (the kernels of the descriptor -> tiles), Scheme A:
+//   FP32, one step per pass    60^2      301^2     400^2     500^2     600^2
+//     extrapolated walls    4.6 -> 1.6  6.2 -> 3.7  6.3 -> 4.7  8.3 -> 6.3  8.5 -> 9.1
+//     periodic              4.1 -> 1.6  4.5 -> 2.9  6.2 -> 3.7  6.2 -> 5.3
+//   FP32, two steps per pass
+//     extrapolated walls    6.2 -> 1.6  6.2 -> 3.7  7.4 -> 4.7  7.4 -> 6.3  7.3 -> 9.1
+//     periodic              4.1 -> 1.6  4.1 -> 2.9  5.0 -> 3.7  5.1 -> 5.3
+//   FP64, extrapolated      24.6 -> 10.4  55 -> 43  81 -> 72  104 -> 96
+// A periodic lattice with two steps per pass keeps its two-step kernel from 130,000 nodes
+// on (Scheme A 170,000), where a call of two steps (400^2 Scheme B 8.2 us) is one launch over
+// the tiles (10.3). Not mended by this choice: calls of one or two single steps on periodic
+// lattices, 301^2 Scheme A 4.5 -> 6.1 and 500^2 6.2 -> 8.2 us per step, where longer calls gain. FP64 Scheme B
+// without walls keeps the one-step kernel where one step per launch over the tiles takes as
+// many turns of the FP64 pipe: 250^2 20.5 us against 22.6.
 static bool tile_general_wanted(lbm_solver *s, int sms)
 {
-    if (s->fixed || s->d.kernel_variant != 0 || s->d.block_rows != 0 || s->c.cfree || s->d.prec == LBM_BF16S || s->c.conv > 2) return false;
-    if ((long long)s->d.nx * s->d.ny > (s->d.prec == LBM_F64 ? 500000 : 250000)) return false;
+    if (s->fixed || s->d.kernel_variant != 0 || s->d.block_rows != 0 || s->c.cfree || s->d.prec == LBM_BF16S || s->c.conv > 2)
+        return false;
+    const long long n = (long long)s->d.nx * s->d.ny;
+    const bool f64 = s->d.prec == LBM_F64, periodic = s->d.bc_x == LBM_PERIODIC && s->d.bc_y == LBM_PERIODIC;
+    if (n > (f64 ? 500000 : 250000)) return false;
+    if (periodic && s->d.steps_per_pass == 2 && n > (s->d.scheme == LBM_SCHEME_A ? 170000 : 130000)) return false;
     need_plan(s, true, sms);
-    return s->plan.us < 1e29 && (s->d.prec == LBM_F64 || s->plan.T >= 2);
+    if (s->plan.us >= 1e29 || (!f64 && s->plan.T < 2)) return false;
+    if (f64 && periodic && s->d.scheme == LBM_SCHEME_B && s->plan.T == 1) {
+        const int blocks = ((s->d.nx + 31) / 32) * ((s->d.ny + 7) / 8), warps = (s->plan.W * s->plan.H + 31) / 32;
+        return (warps + 3) / 4 < 2 * ((blocks + sms - 1) / sms);
+    }
+    return true;
 }
 
 // FP32 on the path left to the library: the tiles with up to two single steps after them (a
@@ -214,7 +234,8 @@ Route plan_route(lbm_solver *s, int nsteps, int sms)
 {
     Route r;
     if (general_path(s)) {
-        if (tile_general_wanted(s, sms)) r.tiles = fewest_tile_launches(s, nsteps);
+        double us;
+        if (tile_general_wanted(s, sms)) r.tiles = tile_launches(s, nsteps, launch_parity(s, nsteps), 1, &us);
         else if (s->d.steps_per_pass == 2) { r.twos = nsteps / 2; r.ones = nsteps % 2; }
         else r.ones = nsteps;
         return r;

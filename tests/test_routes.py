@@ -148,6 +148,9 @@ MEASURED = [
     (64, 16384, P2, 2, "twos"), (2, 300000, P2, 20, "twos"),
     (128, 16384, W2, 4, "twos"), (121, 20000, P2, 20, "pairs"), (128, 16384, W2, 400, "fours"),
     (4096, 4096, W2, 400, "fours"), (4096, 4096, P2, 2, "pairs"), (1023, 777, {}, 250, "fours"),
+    (450, 450, dict(conv=2, **P2), 20, "twos"), (500, 500, dict(conv=2, **P2), 2, "twos"),
+    (350, 350, dict(conv=2, **P2), 20, "tiles"), (450, 450, dict(conv=2), 20, "tiles"),
+    (250, 250, dict(conv=2, prec="f64"), 20, "ones"), (200, 200, dict(conv=2, prec="f64"), 20, "tiles"),
     (400, 400, {}, 1000, "tiles"), (128, 128, dict(prec="f64"), 1000, "tiles"), (4096, 4096, dict(prec="f64"), 20, "tiles"),
     (16384, 8192, dict(prec="f64"), 20, "ones")]
 
