@@ -325,6 +325,10 @@ typedef struct lbm_ensemble_s *lbm_ensemble;
 
 /* Device workspace bytes for `count` instances of sizes nx[i] x ny[i]. */
 int lbm_ensemble_workspace_size(int count, const int *nx, const int *ny, size_t *bytes);
+/* Pieces of strips of the four-step sweeps (lbm_ensemble_configure) for these sizes;
+   0: these instances take the two-step tiles, being too small or too narrow for
+   strips of 120 columns to be faster. Host only. */
+int lbm_ensemble_strips(int count, const int *nx, const int *ny, int *strips);
 /* Create; coeffs: `count` entries (per-instance u and K). A synchronous set-up
    call: it enqueues the copies of the instance and tile tables into the caller's
    workspace on `stream` and waits for `stream` (no other stream is touched), so
@@ -339,8 +343,8 @@ int lbm_ensemble_set_phi(lbm_ensemble e, const void *dev_phi, int prec, void *st
 /* Persistent launches advance 1 (default) or 2 time steps each; with 2, every
    launch runs a two-step shared-memory tile routine on the tiles of all
    instances (two steps per sweep through HBM); with the default grid and tiles
-   below, and instances of 16 nodes a side or more, an even number of the launches
-   of a call advance four steps each instead, the states being equal bit for bit.
+   below, and instances for which lbm_ensemble_strips is not 0, an even number of the
+   launches of a call advance four steps each instead, the states being equal bit for bit.
    Set before capturing a graph. */
 int lbm_ensemble_configure(lbm_ensemble e, int steps_per_pass);
 /* Grid of the two-step launches: persistent = 0 (default) launches one block

@@ -101,6 +101,7 @@ SIGNATURES = {
     "lbm3_reduce": [_VP, _VP, _VP, _VP],
     "lbm3_debug_flags": [_VP, ctypes.POINTER(_I), _VP],
     "lbm_ensemble_workspace_size": [_I, _VP, _VP, ctypes.POINTER(_SZ)],
+    "lbm_ensemble_strips": [_I, _VP, _VP, ctypes.POINTER(_I)],
     "lbm_ensemble_create": [ctypes.POINTER(_VP), _I, _VP, _VP, _VP, _VP, _SZ, _VP],
     "lbm_ensemble_destroy": [_VP],
     "lbm_ensemble_info": [_VP, ctypes.POINTER(ctypes.c_longlong), ctypes.POINTER(_I), ctypes.POINTER(_I)],

@@ -52,8 +52,20 @@ int ens_layout(int count, const int *nx, const int *ny, EnsLayout *L)
     // against 35.2, 14 M nodes 78.0 against 104.8
     if (strip_rows * kEns4Cols < 4000000) fits4 = false;
     L->rows4 = (int)std::min(128LL, std::max(32LL, strip_rows / 1824));
-    for (int i = 0; i < count && fits4; ++i)
-        items4 += (long long)((nx[i] + kEns4Cols - 1) / kEns4Cols) * ((ny[i] + L->rows4 - 1) / L->rows4);
+    // a strip's iteration costs the same however few of its 120 columns an instance fills: the
+    // iterations of the strips, four steps, against the 30 x 30 tiles of two sweeps of two. us
+    // per step of tiles / strips, and iterations per tile: 4000 of 16^2 22.7 / 48.1, 25.0; 300 of
+    // 20 x 1000 86.7 / 158, 31.5; 3000 of 40^2 66.2 / 71.5, 12.3; 300 of 128^2 43.1 / 43.7, 13.1; 300 of
+    // 121^2 45.0 / 46.0, 12.0; 1000 of 64^2 49.2 / 43.6, 9.1; 600 of 100^2 59.3 / 42.5, 8.5; 40 of 500^2
+    // 72.3 / 53.3, 10.2; 256 of 64 to 1023 511 / 325
+    long long iterations = 0;
+    for (int i = 0; i < count && fits4; ++i) {
+        const long long strips = (nx[i] + kEns4Cols - 1) / kEns4Cols;
+        const int chunks = (ny[i] + L->rows4 - 1) / L->rows4, H = (ny[i] + chunks - 1) / chunks;
+        items4 += strips * chunks;
+        iterations += strips * chunks * (H + 9);
+    }
+    if (2 * iterations > 23 * tiles2) items4 = 0;
     L->nitems4 = (int)items4;
     size_t off = 0;
     L->off_inst = off;
@@ -106,6 +118,15 @@ int lbm_ensemble_workspace_size(int count, const int *nx, const int *ny, size_t 
     EnsLayout L;
     if (int rc = ens_layout(count, nx, ny, &L)) return rc;
     *bytes = L.total;
+    return LBM_OK;
+}
+
+int lbm_ensemble_strips(int count, const int *nx, const int *ny, int *strips)
+{
+    if (!strips) return fail(LBM_EINVAL, "null strip count");
+    EnsLayout L;
+    if (int rc = ens_layout(count, nx, ny, &L)) return rc;
+    *strips = L.nitems4;
     return LBM_OK;
 }
 

@@ -163,6 +163,20 @@ def test_the_route_is_the_measured_one(nx, ny, kw, steps, kernel, sms):
     assert max(r, key=lambda k: r[k] * per[k]) == kernel, r
 
 
+@pytest.mark.parametrize("sizes,strips", [
+    ([(16, 16)] * 4000, False), ([(40, 40)] * 3000, False), ([(20, 1000)] * 300, False),
+    ([(16 + i % 49, 16 + (7 * i) % 49) for i in range(3000)], False), ([(2000, 15), (2000, 2000)], False),
+    ([(64, 64)] * 1000, True), ([(100, 100)] * 600, True), ([(1000, 20)] * 300, True), ([(500, 500)] * 40, True),
+    ([(4096, 4096)], True), ([(1000, 1000)], False)])
+def test_ensembles_take_strips_where_they_are_faster(sizes, strips):
+    n = len(sizes)
+    nx, ny = (ctypes.c_int * n)(*[a for a, _ in sizes]), (ctypes.c_int * n)(*[b for _, b in sizes])
+    v = ctypes.c_int(-1)
+    assert C.lib().lbm_ensemble_strips(n, nx, ny, ctypes.byref(v)) == C.LBM_OK
+    assert (v.value > 0) == strips, v.value
+    assert C.lib().lbm_ensemble_strips(n, nx, ny, None) == C.LBM_EINVAL
+
+
 def test_route_arguments_are_checked():
     s = Lattice(64, 64)
     v = (ctypes.c_int * 5)()
