@@ -430,13 +430,25 @@ cudaError_t launch_sweep3(const lbm3_solver *s, bool prepare, cudaStream_t st)
     return cudaErrorInvalidValue;
 }
 
-// FP32, periodic, launch left to the library (block_rows 0), and large enough (the
-// figures stand at the kernel); 32-bit byte offsets within a slab.
+// FP32, periodic, launch left to the library (block_rows 0), large enough (the figures
+// stand at the kernel), 32-bit byte offsets within a slab, and estimated faster. A plane of a
+// 30 x 14 column costs a block the same time but for its traffic, however little of it a
+// flat or narrow lattice fills, and a chunk of 16 planes the first step on two more; a one-step
+// warp of 32 nodes costs what HBM takes, more on rows that are no multiple of it (ns). us per step of single
+// steps / sweeps: 256^3 376 / 274, 64 x 64 x 1024 96 / 89, 31 x 31 x 4400 162 / 128, 8 x 9 x 65535 399 / 265,
+// 61 x 29 x 2400 129 / 118, 96 x 15 x 3000 101 / 118, 32 x 15 x 8800 99 / 149, 4096 x 2 x 512 96 / 255.
 bool sweep3_wanted(const lbm3_solver *s)
 {
-    return s->d.prec == LBM_F32 && s->d.block_rows == 0 && s->d.bc[0] == LBM_PERIODIC && s->d.bc[1] == LBM_PERIODIC &&
-           s->d.bc[2] == LBM_PERIODIC && (long long)s->d.nx * s->d.ny * s->d.nz >= (1LL << 22) &&
-           s->pitch * s->d.ny < (1LL << 29) && (s->d.ny + 13) / 14 <= 65535;
+    if (!(s->d.prec == LBM_F32 && s->d.block_rows == 0 && s->d.bc[0] == LBM_PERIODIC && s->d.bc[1] == LBM_PERIODIC &&
+          s->d.bc[2] == LBM_PERIODIC && (long long)s->d.nx * s->d.ny * s->d.nz >= (1LL << 22) &&
+          s->pitch * s->d.ny < (1LL << 29) && (s->d.ny + 13) / 14 <= 65535))
+        return false;
+    const double columns = (double)((s->d.nx + kS3X - 1) / kS3X) * ((s->d.ny + 13) / 14);
+    const double fill = (double)s->d.nx * s->d.ny / (columns * kS3X * 14);
+    const double sweep = 1.05 * columns * (s->d.nz * (6.3 + 5.6 * fill) + 12.0 * ((s->d.nz + 15) / 16));
+    const double warps = (double)((s->d.nx + 31) / 32) * s->d.ny * s->d.nz;
+    const double ones = 2.0 * warps * (s->d.nx < 64 && s->d.nx % 32 ? 0.95 : 0.74);
+    return sweep < ones;
 }
 
 template <int PREC>

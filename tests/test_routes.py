@@ -177,6 +177,21 @@ def test_ensembles_take_strips_where_they_are_faster(sizes, strips):
     assert C.lib().lbm_ensemble_strips(n, nx, ny, None) == C.LBM_EINVAL
 
 
+@pytest.mark.parametrize("size,sweeps", [
+    ((256, 256, 256), True), ((64, 64, 1024), True), ((31, 31, 4400), True), ((61, 29, 2400), True), ((240, 210, 96), True),
+    ((4096, 512, 2), True), ((96, 15, 3000), False), ((32, 15, 8800), False), ((4096, 2, 512), False), ((128, 128, 128), False)])
+def test_d3q19_sweeps_where_they_are_faster(size, sweeps):
+    L = C.lib()
+    d, n, h, v = C.Desc3(), ctypes.c_size_t(), ctypes.c_void_p(), (ctypes.c_int * 2)()
+    d.nx, d.ny, d.nz, d.prec = *size, C.LBM_F32
+    C.check(L.lbm3_workspace_size(ctypes.byref(d), ctypes.byref(n)))
+    C.check(L.lbm3_create(ctypes.byref(h), ctypes.byref(d), ctypes.c_void_p(1 << 20), n.value))
+    for steps in (0, 1, 3, 4, 7, 40):
+        C.check(L.lbm3_step_route(h, steps, v))
+        assert list(v) == ([steps // 4 * 2, steps % 4] if sweeps else [0, steps])
+    L.lbm3_destroy(h)
+
+
 def test_route_arguments_are_checked():
     s = Lattice(64, 64)
     v = (ctypes.c_int * 5)()
