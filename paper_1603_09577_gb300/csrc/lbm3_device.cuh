@@ -174,15 +174,17 @@ struct Params3 {
 };
 
 // With walls: feq_k + feq_opp(k) at the wall of direction k = 1..18, by the set of axes
-// whose walls its link crosses (bit a: axis a; the mean value of the walls). Only the
-// kernels that read it take it: up to a kilobyte of kernel arguments per launch (periodic
-// FP64, host time per launch 2.39 us with it, 2.02 before there was a table).
+// whose walls its link crosses (bit a: axis a; the mean value of the walls). Periodic FP64
+// and FP32 kernels go without: up to a kilobyte of kernel arguments per launch (FP64, host
+// time per launch 2.39 us with it, 2.12 without). BF16S does not read it either, but with
+// shorter arguments the compiler schedules that kernel otherwise: 256 x 256 x 128 with walls and
+// cubic diffusion 197 us against 180, quadratic flux 188 against 177.
 template <class C>
 struct Params3W : Params3<C> {
     C wt[18][7];
 };
 template <int PREC, bool WALLS>
-using StepParams3 = std::conditional_t<WALLS && PREC != LBM_BF16S, Params3W<typename St3<PREC>::C>,
+using StepParams3 = std::conditional_t<WALLS || PREC == LBM_BF16S, Params3W<typename St3<PREC>::C>,
                                        Params3<typename St3<PREC>::C>>;
 
 // Coefficients at phi (Eq. 7 families, D = g(phi) I): B, B', the tensor
