@@ -234,7 +234,8 @@ int lbm_reduce(lbm_handle h, const double *dev_ref, double *dev_out, void *strea
 
 /* Failure detection: counts the nodes whose phi(t_n) is not finite (a blown-up
    run, a NaN in the input). Synchronises `stream`. Returns LBM_ENONFINITE (and
-   the count in *nonfinite, which may be NULL) if there is any, else LBM_OK. */
+   the count in *nonfinite, which may be NULL) if there is any, LBM_ETIMEOUT if a
+   kernel's bounded wait for its input ran out since lbm_set_phi, else LBM_OK. */
 int lbm_check_finite(lbm_handle h, long long *nonfinite, void *stream);
 
 /* Checked builds (liblbm_checked.so, compiled with LBM_CHECKED): every node
@@ -257,6 +258,11 @@ int lbm_build_checked(void);
    `stream`. The staged kernel reports the same condition by OR-ing 16 into the
    word lbm_debug_flags reads. */
 int lbm_debug_wait_probe(unsigned polls, int *dev_status, void *stream);
+/* late = 1: the four-step sweeps of this handle take their copies of input for late, for
+   tests of what follows: a sweep whose bounded wait runs out sets 16 in the word of
+   lbm_debug_flags, leaves NaN where the input is missing, and ends in bounded time;
+   lbm_check_finite then returns LBM_ETIMEOUT. */
+int lbm_debug_late_copies(lbm_handle h, int late);
 
 /* Rate probe of the FP64 pipe, the roof of the LBM_F64 step kernel (the paper has
    no counterpart: it is a measurement aid). Launches blocks x threads threads,

@@ -79,6 +79,7 @@ SIGNATURES = {
     "lbm_reduce_field_noalloc": [_VP, _VP, ctypes.c_longlong, _VP, _VP],
     "lbm_check_finite": [_VP, ctypes.POINTER(ctypes.c_longlong), _VP],
     "lbm_debug_flags": [_VP, ctypes.POINTER(_I), _VP],
+    "lbm_debug_late_copies": [_VP, _I],
     "lbm_build_checked": [],
     "lbm_debug_wait_probe": [ctypes.c_uint, _VP, _VP],
     "lbm_probe_fp64": [_I, _I, _I, _VP, ctypes.POINTER(ctypes.c_longlong), _VP],

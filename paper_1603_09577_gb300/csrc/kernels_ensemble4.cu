@@ -47,6 +47,7 @@ k_ens_march(const EnsInst *__restrict__ inst, const int4 *__restrict__ items, in
     a.ny = I.ny;
     a.abb_x = a.abb_y = 0;
     a.has_src = 0;
+    a.give_up = 0;
     a.err = I.err;
     const bool cols = it.y - kE4T < 0 || it.y - (kE4T - 1) + E4::kW >= a.nx || it.y - kE4T + E4::kInW > a.pitch;
     if (cols) march_strip<CONV, DIFF, 0, false, kE4T, kE4KW, kE4P, kE4Stage, true>(a, kc, sm_e4, it.y, it.z, it.w, true, false);

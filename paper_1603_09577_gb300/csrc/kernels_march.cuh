@@ -47,6 +47,7 @@ struct MarchArgs {
     int abb_x, abb_y;
     float wt[8][3];            // wall terms (Params)
     int has_src;
+    int give_up;               // 1: level 0 takes its first row for late (a test of what follows)
     int *err;
 };
 
@@ -84,9 +85,9 @@ __device__ __forceinline__ void bulk_copy(unsigned to, const float *from, unsign
                  : "memory");
 }
 // bounded wait for phase `parity`; false when the limit ran out
-__device__ __forceinline__ bool march_wait(unsigned bar, unsigned parity)
+__device__ __forceinline__ bool march_wait(unsigned bar, unsigned parity, unsigned polls = 1u << 20)
 {
-    for (unsigned i = 0; i < (1u << 20); ++i) {
+    for (unsigned i = 0; i < polls; ++i) {
         unsigned done;
         asm volatile("{\n\t.reg .pred p;\n\t"
                      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
@@ -242,15 +243,12 @@ __device__ __forceinline__ void march_strip(const MarchArgs &a, const Coll<F2> &
     if (lev == 0) {
         auto column = [&](int x) { return a.abb_x ? min(max(x, 0), a.nx - 1) : wrap_index(x, a.nx); };
         unsigned phases = 0;                             // bit j: the phase slot j's next row completes
-        bool late = false;
-        int use = 0;
+        int use = 0, i = 0, r = r_first;
+        const int n_run = a.give_up ? 0 : n_it;
         march_barrier(M::kThreads);
-        for (int i = 0, r = r_first; i < n_it; ++i, ++r) {
+        for (; i < n_run; ++i, ++r) {
             if (r >= lo && r <= hi) {
-                if (!late && !march_wait(bars_s + 8 * use, (phases >> use) & 1)) {
-                    late = true;                         // the copy did not arrive: report, and wait no more
-                    if (lane == 0) atomicOr(a.err, 16);
-                }
+                if (!march_wait(bars_s + 8 * use, (phases >> use) & 1)) break;
                 phases ^= 1u << use;
                 const float *in = stage + use * M::kInSlot + 2 * q0 + 1;
                 F2 g[P][9];
@@ -282,8 +280,21 @@ __device__ __forceinline__ void march_strip(const MarchArgs &a, const Coll<F2> &
             s3 = ring_next(s3, 3, w4);
             march_barrier(M::kThreads);
         }
-        if (late)                                        // shared memory is given back: wait once more for what is in flight
-            for (int j = 0; j < M::kStage; ++j) march_wait(bars_s + 8 * j, ((phases >> j) & 1) ^ 1);
+        if (i < n_it && lane == 0) atomicOr(a.err, 16);  // a copy did not arrive in time
+        for (; i < n_it; ++i, ++r) {                     // no result from what is not there: NaN from here on
+            if (r >= lo && r <= hi) {                    // (the copies still end before their slots are filled again)
+                march_wait(bars_s + 8 * use, (phases >> use) & 1, 1u << 12);
+                phases ^= 1u << use;
+            }
+            for (int p = 0; p < P; ++p)
+                each_k([&](auto K) {
+                    ring_put<K>(sm + (cy(K) > 0 ? s4 : s3) + ring_plane(K, w4), w4, q0 + 32 * p, F2(__int_as_float(0x7fffffff)));
+                });
+            use = use == M::kStage - 1 ? 0 : use + 1;
+            s4 = ring_next(s4, 4, w4);
+            s3 = ring_next(s3, 3, w4);
+            march_barrier(M::kThreads);
+        }
     } else {
         const bool copier = warp == KW;
         auto plane_cy = [](int k) { return (k == 2 || k == 5 || k == 6) ? 1 : ((k == 4 || k == 7 || k == 8) ? -1 : 0); };
@@ -446,6 +457,7 @@ static cudaError_t march_t(const lbm_solver *s, int src, bool prepare, cudaStrea
     for (int k = 0; k < 8; ++k)
         for (int z = 0; z < 3; ++z) a.wt[k][z] = p.wt[k][z];
     a.has_src = p.has_src;
+    a.give_up = s->give_up;
     a.err = p.err;
     static_assert(M::kOut == kMarchOut, "strips of the launch's grid");
     const MarchGrid g = march_grid(p.nx, p.ny, s->sms);

@@ -568,9 +568,13 @@ int lbm_check_finite(lbm_handle h, long long *nonfinite, void *stream)
     double out[8];
     if (int rc = cuda_check(cudaMemcpyAsync(out, h->check, sizeof(out), cudaMemcpyDeviceToHost, st), "lbm_check_finite copy"))
         return rc;
+    int flags = 0;
+    if (int rc = cuda_check(cudaMemcpyAsync(&flags, h->err, sizeof(int), cudaMemcpyDeviceToHost, st), "lbm_check_finite flags"))
+        return rc;
     if (int rc = cuda_check(cudaStreamSynchronize(st), "lbm_check_finite sync")) return rc;
     const long long bad = (long long)out[6];
     if (nonfinite) *nonfinite = bad;
+    if (flags & 16) return fail(LBM_ETIMEOUT, "a kernel's bounded wait for its input ran out: the state is not valid");
     if (bad) return fail(LBM_ENONFINITE, std::to_string(bad) + " nodes have a non-finite phi at step " + std::to_string(h->t));
     return LBM_OK;
 }
@@ -583,6 +587,14 @@ int lbm_debug_flags(lbm_handle h, int *flags, void *stream)
     if (int rc = cuda_check(cudaMemcpyAsync(flags, h->err, sizeof(int), cudaMemcpyDeviceToHost, st), "lbm_debug_flags"))
         return rc;
     return cuda_check(cudaStreamSynchronize(st), "lbm_debug_flags sync");
+}
+
+int lbm_debug_late_copies(lbm_handle h, int late)
+{
+    if (check_handle(h)) return LBM_EINVAL;
+    if (late != 0 && late != 1) return fail(LBM_EINVAL, "late must be 0 or 1");
+    h->give_up = late;
+    return LBM_OK;
 }
 
 int lbm_build_checked(void)

@@ -76,6 +76,7 @@ struct lbm_solver {
     double *check = nullptr;        // 8 doubles: reduction output of lbm_check_finite
     int *err = nullptr;             // index-fault word of checked builds
     int cur = 0;
+    int give_up = 0;                // 1: the four-step sweeps take every copy for late (a test)
     int fixed = 0;                  // 1: the kernels that the descriptor names, whatever the size
     int sms = 0;                    // SMs of the device, read at the first step
     lbm::TilePlan plan;
