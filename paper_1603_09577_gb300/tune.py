@@ -1,7 +1,8 @@
 """Autotuner of the launch configuration of one lattice.
 
 For a problem (grid, storage precision, walls, coefficient family) it times the
-candidate configurations on the current device -- kernel variant (one node or
+candidate configurations on the current device -- the launch left to the library
+(kernel_variant 0, block_rows 0), kernel variant (one node or
 four x-adjacent nodes per thread), rows per thread block, one or two time steps
 per sweep through memory (shared-memory tiles of one or two nodes per thread,
 the register column march with 16 to 128 rows per warp, the TMA-staged tile) --
@@ -34,6 +35,8 @@ import torch
 from .solver import Solver
 
 _lock = threading.Lock()
+# part of every cache key: entries of kernels and candidates that have changed are timed again
+_VERSION = 2
 
 
 def cache_path() -> str:
@@ -43,7 +46,7 @@ def cache_path() -> str:
 
 def _key(nx, ny, prec, bc, conv, diff, per_cell_K, scheme="B"):
     dev = torch.cuda.get_device_name()
-    return f"{dev}|{nx}x{ny}|{prec}|{bc[0]},{bc[1]}|c{conv}d{diff}|K{int(per_cell_K)}|s{scheme}"
+    return f"{dev}|{nx}x{ny}|{prec}|{bc[0]},{bc[1]}|c{conv}d{diff}|K{int(per_cell_K)}|s{scheme}|v{_VERSION}"
 
 
 def _general(bc, conv, diff, scheme) -> bool:
@@ -51,16 +54,18 @@ def _general(bc, conv, diff, scheme) -> bool:
 
 
 def general_candidates(prec: str, per_cell_K: bool):
-    """The general kernels: one node per thread (rows per block), and for FP32
-    with constant K the two-step tile kernel."""
-    out = [dict(kernel_variant=1, block_rows=b, steps_per_pass=1) for b in (1, 2, 4, 8)]
+    """The general kernels: the library's choice, one node per thread (rows per block),
+    and for FP32 with constant K two steps per pass."""
+    out = [dict(kernel_variant=0, block_rows=0, steps_per_pass=1)]
+    out += [dict(kernel_variant=1, block_rows=b, steps_per_pass=1) for b in (1, 2, 4, 8)]
     if prec == "f32" and not per_cell_K:
         out.append(dict(kernel_variant=0, block_rows=0, steps_per_pass=2))
     return out
 
 
 def candidates(nx: int, prec: str):
-    out = [dict(kernel_variant=1, block_rows=b, steps_per_pass=1) for b in (1, 2, 4, 8)]
+    out = [dict(kernel_variant=0, block_rows=0, steps_per_pass=1)]      # the constructor's defaults
+    out += [dict(kernel_variant=1, block_rows=b, steps_per_pass=1) for b in (1, 2, 4, 8)]
     if prec != "f64" and nx % 4 == 0:
         out += [dict(kernel_variant=2, block_rows=b, steps_per_pass=1) for b in (1, 2, 4, 8)]
     if prec != "f64":
@@ -143,7 +148,7 @@ def ensemble_candidates():
 def _ensemble_key(instances, conv, diff):
     sig = hashlib.sha256(json.dumps([[int(d["nx"]), int(d["ny"])] for d in instances]).encode()).hexdigest()[:16]
     dev = torch.cuda.get_device_name()
-    return f"{dev}|ensemble|{len(instances)}|{sig}|c{conv}d{diff}"
+    return f"{dev}|ensemble|{len(instances)}|{sig}|c{conv}d{diff}|v{_VERSION}"
 
 
 def _load(path):
