@@ -12,8 +12,8 @@
 // levels of an iteration are independent and one barrier per iteration is enough.
 //
 // Cost: every population is read and written once per T steps (18 B per update
-// for T = 4 in FP32). The strip gives up T - 1 columns on either side (a strip of
-// 128 columns writes 122), and a chunk of H rows takes H + 3 (T - 1) iterations to
+// for T = 4 in FP32). The strip gives up T - 1 columns on either side, and writes a
+// multiple of four columns (120 of 128), and a chunk of H rows takes H + 3 (T - 1) iterations to
 // fill and drain, in which the other blocks of the SM run.
 //
 // Alignment: level l's pairs start one column right of level l - 1's, so a pull

@@ -1,5 +1,7 @@
 // kernels_tile.cuh -- up to kTileMaxT fused time steps per launch for small lattices
-// (Scheme B): FP64, and FP32 with two x-adjacent nodes per packed instruction.
+// (Scheme B): FP64, and FP32 with two x-adjacent nodes per packed instruction. FP64
+// lattices too large for a second step per launch take it too, one step per launch
+// (route.cu has both sides measured).
 //
 // A launch on a small lattice costs more than its arithmetic: the host's part, the
 // gap to the next launch and the latency of the pulls. Here a block owns a W x H
