@@ -13,8 +13,9 @@ namespace lbm {
 // the statistics: 13,981 -> 12,548 us, the reduction's 32-bit index division included).
 // FP32 and BF16-shifted storage keep the two-stage form and its bits.
 template <int CONV, int DIFF>
-__device__ __forceinline__ void initial_f64(const Coll<double> &k, bool src, double phi, double f[9])
+__device__ __forceinline__ void initial_f64(const Params<double> &p, double phi, double f[9])
 {
+    const Coll<double> &k = p.k;
     double e = k.ke1 * phi, eps = -k.nkp1 * phi, h = 0.0, beta = phi, cphi = phi;
     if (DIFF == 1) h = phi * phi;
     if (CONV == 1 || DIFF == 2) h += k.ke3 * phi * phi * phi;
@@ -25,13 +26,13 @@ __device__ __forceinline__ void initial_f64(const Coll<double> &k, bool src, dou
     e += h;
     eps -= h;
     double rho = phi, jx = k.bx * beta, jy = k.by * beta;
-    if (src) {
-        const double R = k.r1 * phi + k.r0, S = 0.5 * (CONV == 1 ? R * phi : R);
+    if (p.has_src) {
+        const double R = p.r1 * phi + p.r0, S = 0.5 * (CONV == 1 ? R * phi : R);
         rho += 0.5 * R;
         e -= R;
         eps += 0.5 * R;
-        jx += k.ux * S;
-        jy += k.uy * S;
+        jx += p.ux * S;
+        jy += p.uy * S;
     }
     const double pxx = -0.25 * k.nkxx * cphi, pxy = -0.25 * k.nkxy * cphi;
     const double r = rho * (1.0 / 9.0), ee = e * (1.0 / 36.0), pp = eps * (1.0 / 36.0);
@@ -62,7 +63,7 @@ k_init(const Params<typename Store<PREC>::C> p, const void *__restrict__ phi_in,
     const C phi0 = in_prec == LBM_F64 ? C(((const double *)phi_in)[in]) : C(((const float *)phi_in)[in]);
     if constexpr (PREC == LBM_F64) {
         C g[9];
-        initial_f64<CONV, DIFF>(p.k, p.has_src != 0, phi0, g);
+        initial_f64<CONV, DIFF>(p, phi0, g);
         S::store_cell(dst, dst_phi, p.plane, (long long)y * p.pitch + x, g, phi0);
         return;
     }

@@ -54,11 +54,11 @@ struct Coll {
     C bx, by, nbx, nby;         // B = b beta (beta = phi, or phi^2 with b = a/2), and -b
     C nkxx, nkxy;               // -(C_xx - C_yy), -C_xy per phi (conv 0) or phi^3 (conv 1)
     C inv_den, phi0;            // Eq. 35: phi = inv_den rho + phi0
-    C r0, r1, ninth;            // R = r0 + r1 phi; 1/9
-    C nhe1, he2;                // source factors of -e and eps
+    C r0, r1;                   // R/9 = r0 + r1 phi
+    C nhe1, he2;                // source factors of -e and eps, per R/9
     C hqx, hqy, hqx2, hqy2;     // of q_x, q_y, and of -2 q_x, -2 q_y
     C jsx, jsy;                 // (I - A/2) B' / 6 of the constant block
-    C ux, uy, sixth, nsixth;    // B' = u (conv 0) or u phi; 1/6, -1/6
+    C ux9, uy9, sixth, nsixth;  // 9 u, B' = u (conv 0) or u phi; 1/6, -1/6
     C four, mtwo, half;         // 4, -2, 1/2
 };
 

@@ -168,13 +168,13 @@ inline Coll<double> make_coll(const lbm_coeffs &c, double A3, double A35, double
     k.nkxy = -third * ux * uy;
     k.inv_den = 1.0 / (1.0 - 0.5 * c.r1);
     k.phi0 = 0.5 * c.r0 * k.inv_den;
-    k.r0 = c.r0; k.r1 = c.r1; k.ninth = 1.0 / 9.0;
-    k.nhe1 = 2.0 * h1 / 36.0; k.he2 = h2 / 36.0;
-    k.hqx = -h4 / 12.0 * ux; k.hqy = -h6 / 12.0 * uy;
-    k.hqx2 = h4 / 6.0 * ux; k.hqy2 = h6 / 6.0 * uy;
-    k.jsx = (1.0 / 6.0 - A3 / 12.0) * ux - A35 / 12.0 * uy;
-    k.jsy = -A35 / 12.0 * ux + (1.0 / 6.0 - A5 / 12.0) * uy;
-    k.ux = ux; k.uy = uy; k.sixth = 1.0 / 6.0; k.nsixth = -1.0 / 6.0;
+    k.r0 = c.r0 / 9.0; k.r1 = c.r1 / 9.0;             // the source's factors below are per R/9
+    k.nhe1 = 2.0 * h1 / 4.0; k.he2 = h2 / 4.0;
+    k.hqx = -0.75 * h4 * ux; k.hqy = -0.75 * h6 * uy;
+    k.hqx2 = 1.5 * h4 * ux; k.hqy2 = 1.5 * h6 * uy;
+    k.jsx = 9.0 * ((1.0 / 6.0 - A3 / 12.0) * ux - A35 / 12.0 * uy);
+    k.jsy = 9.0 * (-A35 / 12.0 * ux + (1.0 / 6.0 - A5 / 12.0) * uy);
+    k.ux9 = 9.0 * ux; k.uy9 = 9.0 * uy; k.sixth = 1.0 / 6.0; k.nsixth = -1.0 / 6.0;
     k.four = 4.0; k.mtwo = -2.0; k.half = 0.5;
     return k;
 }
