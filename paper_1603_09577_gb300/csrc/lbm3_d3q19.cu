@@ -236,13 +236,12 @@ Coll3<double> make_coll3(const lbm3_solver *s)
     k.inv_den = 1.0 / (1.0 - 0.5 * s->c.r1);
     k.phi0 = 0.5 * s->c.r0 * k.inv_den;
     k.r0 = s->c.r0; k.r1 = s->c.r1;
-    if (!quad) {                                      // R = r0 + r1 phi: the source joins the other terms in phi
+    if (!quad) {                                      // R = r0 + r1 phi: the source joins the moments' other terms in phi
         for (int a = 0; a < 3; ++a) {
             k.nb[a] += k.ph[a] * k.r1;
             k.pc[a] = k.ph[a] * k.r0;
         }
         k.tb += k.hse * k.r1;
-        k.xs += k.hse * k.r1;
         k.hr0 = k.hse * k.r0;
     }
     return k;

@@ -133,8 +133,8 @@ struct Coll3 {
     C i18, i36, i3, qi;         // 1/18, 1/36, 1/3; s_e/4 times the isotropic part
     C ea[3], ep[3], em[3];      // even parts per cphi (Params3)
     C inv_den, phi0, r0, r1;
-    // linear flux with a source: R = r0 + r1 phi, so r1's parts are in nb, tb and xs, and what
-    // is left is u/2 r0 and (1 - s_e/2) r0: three operations fewer
+    // linear flux with a source: R = r0 + r1 phi, so r1's parts of the moments are in nb and
+    // tb, and what is left is u/2 r0 and (1 - s_e/2) r0
     C pc[3], hr0;
 };
 

@@ -38,7 +38,10 @@ __device__ __forceinline__ void relax3(const Coll3<C> &k, C f[19])
         vy = vadd(vy, k.pc[1]);
         vz = vadd(vz, k.pc[2]);
         t = vmad(k.tb, phi, k.hr0);
-        X = vmad(k.xs, phi, k.hr0);
+        // R itself, not folded into xs: xs + hse r1 rounded once was an error of the rate that
+        // every step repeated (FP64, 67 x 24 x 77, r1 = -5e-4, 33 steps: 2.4e-15 against
+        // 64-bit references, 3.7e-16 so; 1,666 us and 1,729)
+        X = vmad(k.hse, vmad(k.r1, phi, k.r0), vmul(k.xs, phi));
     } else {
         t = vmul(k.tb, beta);
         X = vmul(k.xs, phi);
